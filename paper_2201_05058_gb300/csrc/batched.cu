@@ -38,8 +38,8 @@ using namespace pcdf::host;
 namespace pcdf {
 namespace {
 
-constexpr int kThreads = 128;
-constexpr int kBands = kThreads / lean::kCols;  // envelope threads per column
+constexpr int kThreads = 128;  // composite launch
+constexpr int kFirst = 256;    // first launch
 constexpr long long kSpinLimit = 1LL << 22;  // x 256 ns sleep: about one second
 
 enum ItemType : int { kRow = 0, kY = 1, kZ = 2, kDyn = 3, kComp = 4 };
@@ -96,14 +96,12 @@ __device__ bool wait_ge(const int *p, int target, int *err)
 __device__ __forceinline__ void run_rows(const BatchEnv &E, int r0, int r1)
 {
     const int lane = threadIdx.x & 31;
-    for (int r = r0 + (threadIdx.x >> 5); r < r1; r += kThreads / 32)
+    for (int r = r0 + (threadIdx.x >> 5); r < r1; r += kFirst / 32)
         full::row_bits_row<0>(E.occ, nullptr, 0, E.nx, E.ny, r, (long long)E.ny * E.nz, E.W, E.bits, E.carry, lane);
 }
 
-// 5 CTAs per SM: the envelope stages' shared memory (up to 42 KB at 320-voxel
-// axes) allows no more, and the register budget that follows keeps spills
-// to a few words
-__global__ void __launch_bounds__(kThreads, 5)
+// 3 CTAs of 8 warps per SM: the tile of a 320-voxel axis takes 62 KB
+__global__ void __launch_bounds__(kFirst, 3)
     k_batched(const BatchEnv *__restrict__ envs, const BatchItem *__restrict__ items, int n_items, int *state,
               int row_rows, int dyn_slices, int comp_t)
 {
@@ -134,20 +132,20 @@ __global__ void __launch_bounds__(kThreads, 5)
             case kRow:
                 run_rows(E, I.a, min(I.a + row_rows, E.ny * E.nz));
                 break;
-            case kY:  // slice I.a, row word I.b
-                full::edt_xy_block<kBands, true>(E.bits, E.carry, E.nx, E.ny, E.nz, E.W, I.b, I.a, E.mid, smem);
+            case kY:  // slice I.a, columns from 64 I.b
+                full::edt_xy_block<true>(E.bits, E.carry, E.nx, E.ny, E.nz, E.W, I.b, I.a, E.mid, smem);
                 break;
             case kZ:
-                full::edt_z_block<kBands, false, true>(E.mid, E.static_sq, nullptr, 0.f, E.nz,
-                                                       (long long)E.nx * E.ny, (long long)I.a, smem, E.colmax);
+                full::edt_z_block<false, true>(E.mid, E.static_sq, nullptr, 0.f, E.nz, (long long)E.nx * E.ny,
+                                               (long long)I.a, E.nx * E.ny % 2 == 0, smem, E.colmax);
                 break;
             case kDyn: {  // time I.a, slices from I.b / 16, column block I.b % 16
-                const int s0 = I.b >> 4, x0 = (I.b & 15) * kThreads;
+                const int s0 = I.b >> 4, x0 = (I.b & 15) * kFirst;
                 for (int s = s0; s < min(s0 + dyn_slices, E.S); ++s) {
                     if (E.rep && E.rep[I.a * E.S + s] != s)
                         continue;  // read from the earlier slice of equal cross-sections
                     comp::dyn_xy_slice(E.caps + (long long)I.a * E.H, E.H, E.nx, E.ny, E.zlo, E.S, I.a, s, E.cap,
-                                       E.dyn, reinterpret_cast<int32_t *>(smem), x0, min(x0 + kThreads, E.nx));
+                                       E.dyn, reinterpret_cast<int32_t *>(smem), x0, min(x0 + kFirst, E.nx));
                     __syncthreads();
                 }
                 break;
@@ -202,10 +200,9 @@ __global__ void __launch_bounds__(kThreads)
 // shared memory words of the first launch's stages, and of a composite item
 size_t smem_words_env(const CompositePlan &p, const pcdf_grid &g, int H)
 {
-    auto col = [](int n) { return (size_t)lean::kCols * (n + (n + 31) / 32); };
-    size_t w = std::max(col(g.ny), col(g.nz));
+    size_t w = std::max(blockmin::tile_words(g.ny), blockmin::tile_words(g.nz));
     if (p.S > 0)
-        w = std::max(w, (size_t)g.ny * (H + 1) + (size_t)p.cap * kThreads);
+        w = std::max(w, (size_t)g.ny * (H + 1) + (size_t)p.cap * kFirst);
     return w;
 }
 size_t smem_words_comp(const CompositePlan &p) { return (size_t)kThreads * (p.S + 2 + (p.S + 31) / 32); }
@@ -237,6 +234,18 @@ void default_tiles(pcdf_batch_tiles &t)
         t.dyn_slices = 1;
     if (t.comp_t <= 0)
         t.comp_t = 1;
+}
+
+// Every batch may use all of the SM's shared memory: the attribute belongs to
+// the kernel, so a limit set by one batch's plan would refuse another's launch.
+template <class K>
+cudaError_t allow_shared(K kernel)
+{
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   227 * 1024 - (int)a.sharedSizeBytes);
 }
 
 int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, pcdf_batch &B)
@@ -310,7 +319,7 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         for (int r = 0; r < nrows; r += B.tiles.row_rows)
             rows.push_back({kRow, e, r, 0});
         D.need[kRow] = (nrows + B.tiles.row_rows - 1) / B.tiles.row_rows;
-        const int nxb = (g.nx + kThreads - 1) / kThreads;  // column blocks of a slice (<= 4)
+        const int nxb = (g.nx + kFirst - 1) / kFirst;  // column blocks of a slice (<= 2)
         for (int t = 0; t < U.T; ++t)
             for (int s = 0; s < p.S; s += B.tiles.dyn_slices)
                 for (int xb = 0; xb < nxb; ++xb)
@@ -318,12 +327,12 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         D.need[kDyn] = U.T * ((p.S + B.tiles.dyn_slices - 1) / B.tiles.dyn_slices) * nxb;
         const long long zcols = (long long)g.nx * g.ny;
         for (int z = 0; z < g.nz; ++z)
-            for (int w = 0; w < D.W; ++w)
-                ys.push_back({kY, e, z, w});
-        D.need[kY] = g.nz * D.W;
-        for (long long c = 0; c < zcols; c += lean::kCols)
+            for (int x = 0; x < g.nx; x += full::kTileCols)
+                ys.push_back({kY, e, z, x / full::kTileCols});
+        D.need[kY] = g.nz * ((g.nx + full::kTileCols - 1) / full::kTileCols);
+        for (long long c = 0; c < zcols; c += full::kTileCols)
             zs.push_back({kZ, e, (int)c, 0});
-        D.need[kZ] = (int)((zcols + lean::kCols - 1) / lean::kCols);
+        D.need[kZ] = (int)((zcols + full::kTileCols - 1) / full::kTileCols);
         // composite items t-fastest within a column block: the blocks of one
         // column range run together and share the static column in L2
         for (long long c = 0; c < zcols; c += kThreads)
@@ -347,15 +356,15 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
     if (B.smem > 227 * 1024 || B.smem_comp > 227 * 1024)
         return fail(PCDF_EINVAL, "an environment needs %zu bytes of shared memory (limit 227 KB)",
                     std::max(B.smem, B.smem_comp));
-    cudaError_t e = cudaFuncSetAttribute(k_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B.smem);
+    cudaError_t e = allow_shared(k_batched);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_batched_comp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B.smem_comp);
+        e = allow_shared(k_batched_comp);
     if (e != cudaSuccess)
         return cuda_fail(e, "batched kernel attributes");
     int dev = 0, sms = 0, per_sm = 0, per_sm_comp = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batched, kThreads, B.smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batched, kFirst, B.smem);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_comp, k_batched_comp, kThreads, B.smem_comp);
     if (e != cudaSuccess)
@@ -472,7 +481,7 @@ int pcdf_batch_run(const pcdf_batch *b, void *workspace, void *stream)
         return cuda_fail(err, "batch counter reset");
     const BatchEnv *desc = (const BatchEnv *)(ws + b->off_desc);
     const BatchItem *items = (const BatchItem *)(ws + b->off_items);
-    k_batched<<<b->blocks, kThreads, b->smem, st>>>(desc, items, b->n_first, state, b->tiles.row_rows,
+    k_batched<<<b->blocks, kFirst, b->smem, st>>>(desc, items, b->n_first, state, b->tiles.row_rows,
                                                    b->tiles.dyn_slices, b->tiles.comp_t);
     err = cudaGetLastError();
     if (err != cudaSuccess)

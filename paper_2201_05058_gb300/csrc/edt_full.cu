@@ -8,14 +8,13 @@
 //   k_row_bits  one warp per row (y, z): the row's occupancy as 32-bit words
 //               (bit l of word w: voxel x = 32 w + l) and, per word, the
 //               nearest occupied and free voxel left of it and right of it.
-//   k_edt_xy    one CTA per (slice z, 32-column word w), kB threads per
-//               column: the 1-D distance along x of every voxel of its 32
-//               columns from the word and its carries, then the y pass by
-//               the run-split banded envelope of lean.cuh.  Output: the
-//               signed 2-D partial field (int32) of the slice.
-//   k_edt_z     one CTA per 32 consecutive columns (x, y) of the partial
-//               field, kB threads per column: the z pass by the same
-//               envelope, with the float field sign(S) sqrt|S| vox.
+//   k_edt_xy    one CTA per (slice z, 64 columns): the 1-D distance along x of
+//               every voxel of its columns from the words and their carries,
+//               then the y pass by the block search of blockmin.cuh.  Output:
+//               the signed 2-D partial field (int32) of the slice.
+//   k_edt_z     one CTA per 64 consecutive columns (x, y) of the partial
+//               field: the z pass by the same search, with the float field
+//               sign(S) sqrt|S| vox.
 // The 1-D row distances never reach memory, so the grid is read once as
 // bytes and the 2-D partial field is written and read once.
 #include <cuda_runtime.h>
@@ -25,17 +24,8 @@
 namespace pcdf {
 namespace {
 
-using lean::kCols;
-
 constexpr int kRowsPerCta = 8;  // k_row_bits: rows (warps) per CTA
-#ifndef PCDF_XY_BANDS
-#define PCDF_XY_BANDS 8
-#endif
-#ifndef PCDF_Z_BANDS
-#define PCDF_Z_BANDS 8
-#endif
-constexpr int kXyBands = PCDF_XY_BANDS;  // envelope threads per column, y pass
-constexpr int kZBands = PCDF_Z_BANDS;    // envelope threads per column, z pass
+constexpr int kThreads = 256;   // k_edt_xy, k_edt_z: 8 warps share the blocks of a tile
 
 template <int kMode>
 __global__ void __launch_bounds__(32 * kRowsPerCta)
@@ -48,35 +38,39 @@ __global__ void __launch_bounds__(32 * kRowsPerCta)
     full::row_bits_row<kMode>(occ, caps.caps, H, nx, ny, row, nrows, W, bits, carry, threadIdx.x & 31, vec4 != 0);
 }
 
-// six CTAs of 256 threads per SM: 42 registers, and the tile (33 KB at 256
-// rows) with the 16-bit band table fits six times
-template <int kB>
-__global__ void __launch_bounds__(kCols * kB, 6)
+// 46 us for a 256^3 map of 60 boxes (85 us with the stack envelopes it
+// replaced), 33 us for 317 x 211 x 97 with speckle: instruction issue (66 %
+// active).  Four CTAs of 64 registers; held to 48 for five it spills (50 us).
+__global__ void __launch_bounds__(kThreads, 4)
     k_edt_xy(const uint32_t *__restrict__ bits, const uint2 *__restrict__ carry, int nx, int ny, int nz, int W,
              int32_t *__restrict__ mid)
 {
-    extern __shared__ uint32_t smem[];
-    full::edt_xy_block<kB, false>(bits, carry, nx, ny, nz, W, blockIdx.x, blockIdx.y, mid, smem);
+    extern __shared__ __align__(16) uint32_t smem[];
+    full::edt_xy_block<false>(bits, carry, nx, ny, nz, W, blockIdx.x, blockIdx.y, mid, smem);
 }
 
-// colmax (nullable): each column's largest value of sq; five CTAs of 256
-// threads per SM (51 registers: held to 42 for six, it spills and is slower)
-template <int kB, bool kSdf>
-__global__ void __launch_bounds__(kCols * kB, 5)
+// colmax (nullable): each column's largest value of sq.  50 us for the 256^3
+// map (105 us before): the 12 bytes per voxel alone take 30 us.
+template <bool kSdf>
+__global__ void __launch_bounds__(kThreads, 4)
     k_edt_z(const int32_t *__restrict__ mid, int32_t *__restrict__ sq, float *__restrict__ sdf, float vox, int n,
-            long long ncols, int32_t *__restrict__ colmax)
+            long long ncols, int vec, int32_t *__restrict__ colmax)
 {
-    extern __shared__ uint32_t smem[];
-    full::edt_z_block<kB, kSdf, false>(mid, sq, sdf, vox, n, ncols, (long long)blockIdx.x * kCols, smem, colmax);
+    extern __shared__ __align__(16) uint32_t smem[];
+    full::edt_z_block<kSdf, false>(mid, sq, sdf, vox, n, ncols, (long long)blockIdx.x * full::kTileCols, vec != 0, smem,
+                                   colmax);
 }
 
+// The tile of the longest axis may exceed the default 48 KB; one value for
+// every launch, so that calls of other threads cannot lower it in between.
 template <class K>
-cudaError_t set_smem(K kernel, size_t bytes)
+cudaError_t allow_tile(K kernel)
 {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(blockmin::tile_words(blockmin::kMaxBlocks * blockmin::kBlk) * sizeof(uint32_t)));
 }
 
-size_t tile_bytes(int n) { return (size_t)kCols * (n + (n + 31) / 32) * sizeof(uint32_t); }
+size_t tile_bytes(int n) { return blockmin::tile_words(n) * sizeof(uint32_t); }
 
 }  // namespace
 
@@ -119,23 +113,26 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
         return e;
 
     const size_t sxy = tile_bytes(ny);
-    if ((e = set_smem(k_edt_xy<kXyBands>, sxy)) != cudaSuccess)
+    if ((e = allow_tile(k_edt_xy)) != cudaSuccess)
         return e;
-    k_edt_xy<kXyBands><<<dim3((unsigned)W, (unsigned)nz), kCols * kXyBands, sxy, st>>>(bits, carry, nx, ny, nz, W, mid);
+    const unsigned nt = (unsigned)((nx + full::kTileCols - 1) / full::kTileCols);
+    k_edt_xy<<<dim3(nt, (unsigned)nz), kThreads, sxy, st>>>(bits, carry, nx, ny, nz, W, mid);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
 
     const long long ncols = (long long)nx * ny;
-    const unsigned nbz = (unsigned)((ncols + kCols - 1) / kCols);
+    const unsigned nbz = (unsigned)((ncols + full::kTileCols - 1) / full::kTileCols);
     const size_t sz = tile_bytes(nz);
+    // rows of whole 8-byte pairs: two adjacent columns per lane
+    const int vec = ncols % 2 == 0 && (((uintptr_t)sq | (uintptr_t)sdf) & 7u) == 0;
     if (sdf) {
-        if ((e = set_smem(k_edt_z<kZBands, true>, sz)) != cudaSuccess)
+        if ((e = allow_tile(k_edt_z<true>)) != cudaSuccess)
             return e;
-        k_edt_z<kZBands, true><<<nbz, kCols * kZBands, sz, st>>>(mid, sq, sdf, vox, nz, ncols, colmax);
+        k_edt_z<true><<<nbz, kThreads, sz, st>>>(mid, sq, sdf, vox, nz, ncols, vec, colmax);
     } else {
-        if ((e = set_smem(k_edt_z<kZBands, false>, sz)) != cudaSuccess)
+        if ((e = allow_tile(k_edt_z<false>)) != cudaSuccess)
             return e;
-        k_edt_z<kZBands, false><<<nbz, kCols * kZBands, sz, st>>>(mid, sq, nullptr, vox, nz, ncols, colmax);
+        k_edt_z<false><<<nbz, kThreads, sz, st>>>(mid, sq, nullptr, vox, nz, ncols, vec, colmax);
     }
     return cudaGetLastError();
 }

@@ -1,0 +1,69 @@
+"""The block search of the y and z passes (csrc/blockmin.cuh) where it can go
+wrong: tiles of 64 columns and blocks of 8 elements with remainders, sides from
+1 to 512, distances on both sides of the 16-bit range (177 voxels), solid maps
+(the other site set), and the float field's root over every squared distance
+of that range."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+pcdf = pytest.importorskip("paper_2201_05058_gb300")
+
+
+def run(occ, vox=0.05):
+    nz, ny, nx = occ.shape
+    sq, sdf = pcdf.build_static_sdf(torch.from_numpy(np.ascontiguousarray(occ)).to("cuda"), scenes.Grid(nx, ny, nz, vox))
+    return sq.cpu().numpy(), sdf.cpu().numpy()
+
+
+def squares(shape, at):
+    z, y, x = np.ogrid[:shape[0], :shape[1], :shape[2]]
+    return ((z - at[0]) ** 2 + (y - at[1]) ** 2 + (x - at[2]) ** 2).astype(np.int32)
+
+
+def check(occ, want):
+    sq, sdf = run(occ)
+    assert np.array_equal(sq, want)
+    assert np.array_equal(sdf.view(np.int32), oracle.sdf_from_sq(want, 0.05).view(np.int32))
+
+
+# one occupied (or, solid, one free) voxel: the answer in closed form, with
+# every sum of three squares up to 177^2 and beyond
+@pytest.mark.parametrize("solid", [False, True])
+@pytest.mark.parametrize("shape,at", [((180, 178, 179), (0, 0, 0)), ((9, 8, 512), (8, 0, 511)), ((512, 7, 65), (0, 3, 64)),
+                                      ((16, 512, 63), (15, 511, 1)), ((1, 300, 300), (0, 299, 0)), ((177, 1, 178), (176, 0, 0))])
+def test_one_voxel(shape, at, solid):
+    occ = np.full(shape, int(solid), np.uint8)
+    occ[at] = 1 - int(solid)
+    want = squares(shape, at)
+    if solid:
+        want = -want
+        want[at] = 1  # the free voxel: its nearest occupied neighbour
+    else:
+        want[at] = -1
+    check(occ, want)
+
+
+@pytest.mark.parametrize("density", [0.0, 0.0005, 0.03, 0.6, 1.0])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (8, 8, 64), (7, 9, 63), (17, 15, 65), (41, 23, 130), (33, 64, 127), (3, 200, 257)])
+def test_random_maps(shape, density):
+    rng = np.random.default_rng(sum(shape) + int(1e4 * density))
+    occ = (rng.random(shape) < density).astype(np.uint8)
+    check(occ, oracle.edt(occ))
+
+
+# far blocks next to near ones: a few voxels in long grids, a thick slab
+@pytest.mark.parametrize("shape", [(24, 400, 66), (400, 24, 66), (20, 30, 470)])
+def test_sparse_and_thick(shape):
+    rng = np.random.default_rng(shape[0])
+    occ = np.zeros(shape, np.uint8)
+    for _ in range(3):
+        occ[tuple(int(rng.integers(0, n)) for n in shape)] = 1
+    check(occ, oracle.edt(occ))
+    occ[:, : shape[1] // 2] = 1
+    check(occ, oracle.edt(occ))
