@@ -49,7 +49,7 @@ struct BatchItem {
 };
 
 struct BatchEnv {
-    int nx, ny, nz, T, H, zlo, S, cap, W;
+    int nx, ny, nz, T, H, zlo, S, W;
     float vox;
     int need[4];  // items of the row, y, z and capsule stages
     int vec;      // 16-byte copies of all-static column blocks allowed
@@ -139,13 +139,13 @@ __global__ void __launch_bounds__(kFirst, 3)
                 full::edt_z_block<false, true>(E.mid, E.static_sq, nullptr, 0.f, E.nz, (long long)E.nx * E.ny,
                                                (long long)I.a, E.nx * E.ny % 2 == 0, smem, E.colmax);
                 break;
-            case kDyn: {  // time I.a, slices from I.b / 16, column block I.b % 16
-                const int s0 = I.b >> 4, x0 = (I.b & 15) * kFirst;
+            case kDyn: {  // time I.a, slices from I.b / 16, columns from 64 (I.b % 16)
+                const int s0 = I.b >> 4;
                 for (int s = s0; s < min(s0 + dyn_slices, E.S); ++s) {
                     if (E.rep && E.rep[I.a * E.S + s] != s)
                         continue;  // read from the earlier slice of equal cross-sections
-                    comp::dyn_xy_slice(E.caps + (long long)I.a * E.H, E.H, E.nx, E.ny, E.zlo, E.S, I.a, s, E.cap,
-                                       E.dyn, reinterpret_cast<int32_t *>(smem), x0, min(x0 + kFirst, E.nx));
+                    full::capsule_xy_block(E.caps + (long long)I.a * E.H, E.H, E.nx, E.ny, E.zlo + s, I.b & 15,
+                                           E.dyn + ((long long)I.a * E.S + s) * E.nx * E.ny, smem);
                     __syncthreads();
                 }
                 break;
@@ -198,11 +198,11 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // shared memory words of the first launch's stages, and of a composite item
-size_t smem_words_env(const CompositePlan &p, const pcdf_grid &g, int H)
+size_t smem_words_env(const CompositePlan &p, const pcdf_grid &g)
 {
     size_t w = std::max(blockmin::tile_words(g.ny), blockmin::tile_words(g.nz));
     if (p.S > 0)
-        w = std::max(w, (size_t)g.ny * (H + 1) + (size_t)p.cap * kFirst);
+        w = std::max(w, dyn_xy_words(g.ny, p.run_rows));
     return w;
 }
 size_t smem_words_comp(const CompositePlan &p) { return (size_t)kThreads * (p.S + 2 + (p.S + 31) / 32); }
@@ -236,18 +236,6 @@ void default_tiles(pcdf_batch_tiles &t)
         t.comp_t = 1;
 }
 
-// Every batch may use all of the SM's shared memory: the attribute belongs to
-// the kernel, so a limit set by one batch's plan would refuse another's launch.
-template <class K>
-cudaError_t allow_shared(K kernel)
-{
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   227 * 1024 - (int)a.sharedSizeBytes);
-}
-
 int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, pcdf_batch &B)
 {
     using namespace pcdf;
@@ -279,7 +267,7 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         if (int rc = plan_composite(&U.grid, U.T, U.H, U.caps, p))
             return rc;
         if (p.S > 0 && !p.fused)
-            return fail(PCDF_EINVAL, "environment %d: capsule stack bound %d too large for the batched kernel", e,
+            return fail(PCDF_EINVAL, "environment %d: capsule row bound %d too large for the batched kernel", e,
                         p.cap);
         const pcdf_grid &g = U.grid;
         const long long V = (long long)g.nx * g.ny * g.nz;
@@ -300,7 +288,7 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         off += align_up(p.ci.size() * sizeof(CapInfo));
         B.off_rep[e] = off;
         off += align_up(p.rep.size());
-        words = std::max(words, smem_words_env(p, g, U.H));
+        words = std::max(words, smem_words_env(p, g));
         words_comp = std::max(words_comp, smem_words_comp(p));
 
         BatchEnv &D = B.desc[e];
@@ -312,14 +300,13 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         D.H = U.H;
         D.zlo = p.zlo;
         D.S = p.S;
-        D.cap = p.cap;
         D.W = (g.nx + 31) / 32;
         D.vox = g.vox;
         const int nrows = g.ny * g.nz;
         for (int r = 0; r < nrows; r += B.tiles.row_rows)
             rows.push_back({kRow, e, r, 0});
         D.need[kRow] = (nrows + B.tiles.row_rows - 1) / B.tiles.row_rows;
-        const int nxb = (g.nx + kFirst - 1) / kFirst;  // column blocks of a slice (<= 2)
+        const int nxb = (g.nx + full::kTileCols - 1) / full::kTileCols;  // column blocks of a slice (<= 8)
         for (int t = 0; t < U.T; ++t)
             for (int s = 0; s < p.S; s += B.tiles.dyn_slices)
                 for (int xb = 0; xb < nxb; ++xb)

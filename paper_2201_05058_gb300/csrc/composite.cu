@@ -3,26 +3,29 @@
 #include <cuda_runtime.h>
 
 #include "composite.cuh"
+#include "edt_full.cuh"
 
 namespace pcdf {
 namespace {
 
-// Columns per CTA of k_dyn_xy: a slice's columns are shared by ceil(nx / 128)
-// CTAs, one column per thread.
-constexpr int kDynCols = 128;
-
-__global__ void __launch_bounds__(128)
+// Partial fields of the capsules: one CTA per (slab slice, 64 columns, t).
+// 8 warps; like k_edt_xy bound by instruction issue.  3 humans on 256^2, 7
+// distinct slices at each of 20 t: 48 us (111 us with an envelope per column
+// and thread, whose serial chain left 8 % of the warps active); 4 humans on
+// 161 x 115, T = 9: 23 us (82 us).
+__global__ void __launch_bounds__(256, 4)
     k_dyn_xy(const __grid_constant__ CapBatch caps, const __grid_constant__ SlabMap map, int H, int nx, int ny,
-             int zlo, int S, int t0, int cap, int32_t *__restrict__ dyn_mid)
+             int zlo, int S, int t0, int32_t *__restrict__ dyn_mid)
 {
-    const int nxb = (nx + kDynCols - 1) / kDynCols;
-    const int s = (int)blockIdx.x / nxb, xb = (int)blockIdx.x % nxb;
+    const int ntile = (nx + full::kTileCols - 1) / full::kTileCols;
+    const int s = (int)blockIdx.x / ntile, w2 = (int)blockIdx.x % ntile;
+    const int t = t0 + (int)blockIdx.y;
     // a slice whose cross-sections equal an earlier slice's is read from that one
-    if (map.on && map.rep[(t0 + (int)blockIdx.y) * S + s] != s)
+    if (map.on && map.rep[t * S + s] != s)
         return;
-    extern __shared__ __align__(16) int32_t sm[];
-    comp::dyn_xy_slice(caps.caps + blockIdx.y * H, H, nx, ny, zlo, S, t0 + (int)blockIdx.y, s, cap, dyn_mid, sm,
-                       xb * kDynCols, min((xb + 1) * kDynCols, nx));
+    extern __shared__ __align__(16) uint32_t sm[];
+    full::capsule_xy_block(caps.caps + blockIdx.y * H, H, nx, ny, zlo + s, w2,
+                           dyn_mid + ((long long)t * S + s) * nx * ny, sm);
 }
 
 // CTAs are ordered t-fastest, so the T CTAs of one column block run together
@@ -66,26 +69,21 @@ __global__ void k_broadcast_static(const int32_t *__restrict__ static_sq, long l
     }
 }
 
-constexpr int kDynThreads = 128;
-
-size_t dyn_xy_smem(int ny, int H, int cap) { return ((size_t)ny * (H + 1) + (size_t)cap * kDynThreads) * 4; }
-
 }  // namespace
 
-bool dyn_xy_fits(int ny, int H, int cap) { return dyn_xy_smem(ny, H, cap) <= 200 * 1024; }
+size_t dyn_xy_words(int ny, int run_rows) { return blockmin::tile_words(ny) + (size_t)run_rows; }
 
 cudaError_t launch_dyn_xy(const CapBatch *caps, const SlabMap *map, int H, int nx, int ny, int zlo, int S, int t0,
-                          int n_t, int cap, int32_t *dyn_mid, cudaStream_t stream)
+                          int n_t, int run_rows, int32_t *dyn_mid, cudaStream_t stream)
 {
     if (S <= 0 || n_t <= 0)
         return cudaSuccess;
-    const size_t smem = dyn_xy_smem(ny, H, cap);
-    cudaError_t e = cudaFuncSetAttribute(k_dyn_xy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k_dyn_xy);
     if (e != cudaSuccess)
         return e;
-    const unsigned nxb = (unsigned)((nx + kDynCols - 1) / kDynCols);
-    k_dyn_xy<<<dim3((unsigned)S * nxb, (unsigned)n_t), kDynThreads, smem, stream>>>(*caps, *map, H, nx, ny, zlo, S,
-                                                                                     t0, cap, dyn_mid);
+    const unsigned nt = (unsigned)((nx + full::kTileCols - 1) / full::kTileCols);
+    k_dyn_xy<<<dim3((unsigned)S * nt, (unsigned)n_t), 256, dyn_xy_words(ny, run_rows) * 4, stream>>>(
+        *caps, *map, H, nx, ny, zlo, S, t0, dyn_mid);
     return cudaGetLastError();
 }
 

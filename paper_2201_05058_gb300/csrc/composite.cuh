@@ -6,9 +6,9 @@
 // inside their capsules; its sites all lie in the z-slab [zlo, zlo + S) that
 // the capsules touch.  Two kernels build the composite of every t:
 //
-//  k_dyn_xy      one CTA per (slab slice, t): the exact x-interval of each
-//                capsule on every row of the slice, then per column x the
-//                y lower envelopes of the row distances to those intervals.
+//  k_dyn_xy      one CTA per (slab slice, 64 columns, t): the exact x-interval
+//                of each capsule on every row of the slice, then the y pass
+//                of the static EDT (capsule_xy_block in edt_full.cuh).
 //                Output: the 2-D partial field of the slice (signed int32),
 //                with no row-pass intermediate in memory.
 //  k_colmax     the largest static value of every column (x, y).
@@ -35,200 +35,6 @@
 namespace pcdf {
 namespace comp {
 
-
-// ---------------------------------------------------------------------------
-// k_dyn_xy
-// ---------------------------------------------------------------------------
-// Shared memory: rows[ny][H + 1] = interval count, then the merged maximal
-// occupied runs of the row as (xa << 16 | xb); then a stack of `cap` words per
-// thread, laid out [entry][thread].
-
-__device__ __forceinline__ bool row_inside(const int32_t *r, int x)
-{
-    const int cnt = r[0];
-    for (int i = 1; i <= cnt; ++i)
-        if (x >= (r[i] >> 16) && x <= (r[i] & 0xFFFF))
-            return true;
-    return false;
-}
-
-// squared distance along the row from x to the nearest occupied voxel (-1: none)
-__device__ __forceinline__ int row_g_occ(const int32_t *r, int x)
-{
-    const int cnt = r[0];
-    if (cnt == 0)
-        return -1;
-    int d = 1 << 20;
-    for (int i = 1; i <= cnt; ++i) {
-        const int a = r[i] >> 16, b = r[i] & 0xFFFF;
-        const int di = x < a ? a - x : (x > b ? x - b : 0);
-        d = min(d, di);
-    }
-    return d * d;
-}
-
-// squared distance along the row from an occupied x to the nearest free voxel
-// (-1: the whole row is occupied); runs are maximal, so the neighbours of the
-// run holding x are free
-__device__ __forceinline__ int row_g_free(const int32_t *r, int x, int nx)
-{
-    const int cnt = r[0];
-    for (int i = 1; i <= cnt; ++i) {
-        const int a = r[i] >> 16, b = r[i] & 0xFFFF;
-        if (x >= a && x <= b) {
-            int d = 1 << 20;
-            if (a - 1 >= 0)
-                d = x - a + 1;
-            if (b + 1 <= nx - 1)
-                d = min(d, b - x + 1);
-            return d == (1 << 20) ? -1 : d * d;
-        }
-    }
-    return 0;
-}
-
-// The CTA computes columns [x0, x1) of slab slice s of time t (the capsules'
-// runs of every row of the slice are found first; several CTAs can share a
-// slice by its columns).  caps_t: the H capsules of t; sm: ny * (H + 1) +
-// cap * blockDim.x words.
-__device__ __forceinline__ void dyn_xy_slice(const CapInfo *caps_t, int H, int nx, int ny, int zlo, int S, int t,
-                                             int s, int cap, int32_t *__restrict__ dyn_mid, int32_t *sm, int x0,
-                                             int x1)
-{
-    __shared__ int s_ylo, s_yhi;
-    __shared__ uint32_t s_rowbits[(PCDF_MAX_DIM + 31) / 32];  // rows holding a run
-    const int z = zlo + s;
-    const int nthr = blockDim.x, tid = threadIdx.x;
-    const int rw = H + 1;
-    int32_t *rows = sm;
-    uint32_t *stk = reinterpret_cast<uint32_t *>(sm + ny * rw) + tid;  // entry q at stk[q * nthr]
-    if (tid == 0) {
-        s_ylo = ny;
-        s_yhi = -1;
-    }
-    for (int w = tid; w < (ny + 31) / 32; w += nthr)
-        s_rowbits[w] = 0;
-    __syncthreads();
-
-    // rows: merged occupied runs of every capsule crossing this slice
-    for (int y = tid; y < ny; y += nthr) {
-        int32_t *r = rows + y * rw;
-        int cnt = 0;
-        for (int h = 0; h < H; ++h) {
-            const CapInfo &ci = caps_t[h];
-            if (ci.lo[0] > ci.hi[0] || z < ci.lo[2] || z > ci.hi[2] || y < ci.lo[1] || y > ci.hi[1])
-                continue;
-            // the capsule is convex, so its voxels on this row form one run
-            int xa = -1, xb = -2;
-            for (int x = ci.lo[0]; x <= ci.hi[0]; ++x) {
-                if (capsule_contains(ci, x, y, z)) {
-                    if (xa < 0)
-                        xa = x;
-                    xb = x;
-                } else if (xa >= 0) {
-                    break;
-                }
-            }
-            if (xa < 0)
-                continue;
-            int i = cnt;
-            while (i > 0 && (r[i] >> 16) > xa) {
-                r[i + 1] = r[i];
-                --i;
-            }
-            r[i + 1] = (xa << 16) | xb;
-            ++cnt;
-        }
-        int m = 0;  // merge overlapping or touching runs
-        for (int i = 1; i <= cnt; ++i) {
-            const int a = r[i] >> 16, b = r[i] & 0xFFFF;
-            if (m > 0 && a <= (r[m] & 0xFFFF) + 1) {
-                if (b > (r[m] & 0xFFFF))
-                    r[m] = (r[m] & ~0xFFFF) | b;
-            } else {
-                r[++m] = r[i];
-            }
-        }
-        r[0] = m;
-        if (m) {
-            atomicMin(&s_ylo, y);
-            atomicMax(&s_yhi, y);
-            atomicOr(&s_rowbits[y >> 5], 1u << (y & 31));
-        }
-    }
-    __syncthreads();
-    const int ylo = s_ylo, yhi = s_yhi;
-    const long long V2 = (long long)nx * ny;
-
-    for (int x = x0 + tid; x < x1; x += nthr) {
-        int32_t *oc = dyn_mid + ((long long)t * S + s) * V2 + x;  // element y at oc[y * nx]
-        if (!PCDF_IN(x, nx) || !PCDF_IN(s, S))
-            continue;
-        if (yhi < 0) {
-            for (int y = 0; y < ny; ++y)
-                oc[(long long)y * nx] = kInf32;
-            continue;
-        }
-        int fo = ny, lo_ = -1;  // first / last occupied row of this column
-        for (int w = ylo >> 5; w <= yhi >> 5; ++w)
-            for (uint32_t b = s_rowbits[w]; b; b &= b - 1) {
-                const int y = (w << 5) + __ffs(b) - 1;
-                if (row_inside(rows + y * rw, x)) {
-                    if (fo == ny)
-                        fo = y;
-                    lo_ = y;
-                }
-            }
-
-        // distances to free voxels at the occupied voxels (set F).  Free rows
-        // matter only next to an occupied row: the nearest free voxel of any
-        // occupied voxel is the first free row out of its run.
-        if (lo_ >= 0) {
-            const int y0 = max(fo - 1, 0), y1 = min(lo_ + 1, ny - 1);
-            EnvBuilder B(stk, nthr, cap);
-            bool prev_occ = false;  // y0 - 1 lies before the first occupied row
-            bool cur_occ = y0 >= ylo && y0 <= yhi && row_inside(rows + y0 * rw, x);
-            for (int y = y0; y <= y1; ++y) {
-                const bool next_occ = y + 1 <= y1 && y + 1 >= ylo && y + 1 <= yhi && row_inside(rows + (y + 1) * rw, x);
-                int g;
-                if (cur_occ)
-                    g = row_g_free(rows + y * rw, x, nx);
-                else
-                    g = (prev_occ || next_occ) ? 0 : -1;
-                prev_occ = cur_occ;
-                cur_occ = next_occ;
-                if (g >= 0)
-                    B.push(y, g);
-            }
-            EnvCursor F(stk, nthr, B.top);
-            for (int y = fo; y <= lo_; ++y) {
-                if (!row_inside(rows + y * rw, x))
-                    continue;
-                const int f = F.eval(y);
-                if (PCDF_IN(y, ny))
-                    oc[(long long)y * nx] = f < 0 ? -kInf32 : -f;
-            }
-        }
-
-        // distances to occupied voxels at the free voxels (set O): sites are
-        // the rows holding a run (g = 0 where x is inside one)
-        EnvBuilder B(stk, nthr, cap);
-        for (int w = ylo >> 5; w <= yhi >> 5; ++w)
-            for (uint32_t b = s_rowbits[w]; b; b &= b - 1) {
-                const int y = (w << 5) + __ffs(b) - 1;
-                B.push(y, row_g_occ(rows + y * rw, x));
-            }
-        EnvCursor O(stk, nthr, B.top);  // B.top >= 0: some row of [ylo, yhi] holds a run
-        // rows before the column's occupied range, the range (skipping its
-        // occupied rows, which set F wrote), rows after it
-        const int ya = min(fo, ny), yb = lo_ >= 0 ? lo_ + 1 : ny;
-        O.fill(0, ya, oc, nx);
-        for (int y = ya; y < yb; ++y)
-            if (!row_inside(rows + y * rw, x) && PCDF_IN(y, ny))
-                oc[(long long)y * nx] = O.eval(y);
-        O.fill(yb, ny, oc, nx);
-    }
-}
 
 // ---------------------------------------------------------------------------
 // k_composite_z

@@ -61,15 +61,6 @@ __global__ void __launch_bounds__(kThreads, 4)
                                    colmax);
 }
 
-// The tile of the longest axis may exceed the default 48 KB; one value for
-// every launch, so that calls of other threads cannot lower it in between.
-template <class K>
-cudaError_t allow_tile(K kernel)
-{
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(blockmin::tile_words(blockmin::kMaxBlocks * blockmin::kBlk) * sizeof(uint32_t)));
-}
-
 size_t tile_bytes(int n) { return blockmin::tile_words(n) * sizeof(uint32_t); }
 
 }  // namespace
@@ -113,7 +104,7 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
         return e;
 
     const size_t sxy = tile_bytes(ny);
-    if ((e = allow_tile(k_edt_xy)) != cudaSuccess)
+    if ((e = allow_shared(k_edt_xy)) != cudaSuccess)
         return e;
     const unsigned nt = (unsigned)((nx + full::kTileCols - 1) / full::kTileCols);
     k_edt_xy<<<dim3(nt, (unsigned)nz), kThreads, sxy, st>>>(bits, carry, nx, ny, nz, W, mid);
@@ -126,11 +117,11 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
     // rows of whole 8-byte pairs: two adjacent columns per lane
     const int vec = ncols % 2 == 0 && (((uintptr_t)sq | (uintptr_t)sdf) & 7u) == 0;
     if (sdf) {
-        if ((e = allow_tile(k_edt_z<true>)) != cudaSuccess)
+        if ((e = allow_shared(k_edt_z<true>)) != cudaSuccess)
             return e;
         k_edt_z<true><<<nbz, kThreads, sz, st>>>(mid, sq, sdf, vox, nz, ncols, vec, colmax);
     } else {
-        if ((e = allow_tile(k_edt_z<false>)) != cudaSuccess)
+        if ((e = allow_shared(k_edt_z<false>)) != cudaSuccess)
             return e;
         k_edt_z<false><<<nbz, kThreads, sz, st>>>(mid, sq, nullptr, vox, nz, ncols, vec, colmax);
     }

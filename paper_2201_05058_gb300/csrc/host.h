@@ -35,7 +35,8 @@ struct CompositePlan {
     int zlo = 0, zhi = -1, S = 0;
     long long slab = 0;  // T * S * nx * ny
     bool fused = false;  // analytic x+y kernel (else row pass + y envelope)
-    int cap = 0;         // its per-thread stack capacity
+    int cap = 0;         // bound on the capsules' rows that decides it
+    int run_rows = 0;    // rows of the capsules' boxes, at most over t
     size_t need = 0;     // workspace bytes
     size_t colmax_off = 0;  // workspace offset of the static column maxima
     std::vector<uint8_t> rep;  // [T][S] first slab slice with the same capsule cross-sections (empty: identity)

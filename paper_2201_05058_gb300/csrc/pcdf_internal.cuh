@@ -131,14 +131,27 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
 cudaError_t launch_envelope_i16(const int16_t *in, int32_t *out, int n, int nx, long long ncols,
                                 long long outer_stride, long long stride, cudaStream_t stream);
 
-// Analytic x+y passes of the capsule field over the slab slices zlo .. zlo+S-1
-// for t = t0 .. t0 + n_t - 1 (capsules of local t at caps->caps[t * H ...]);
-// output dyn_mid[t][s][y][x], signed 2-D partial squared distances.  `cap` is
-// the per-thread stack capacity; dyn_xy_fits tells whether it fits on chip.
-bool dyn_xy_fits(int ny, int H, int cap);
+// Every launch of `kernel` may use all of the SM's shared memory.  The
+// attribute belongs to the kernel, so one value for all calls: a smaller limit
+// set by another thread or plan in between would refuse a launch.
+template <class K>
+cudaError_t allow_shared(K kernel)
+{
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   227 * 1024 - (int)a.sharedSizeBytes);
+}
+
+// x+y passes of the capsule field over the slab slices zlo .. zlo+S-1 for
+// t = t0 .. t0 + n_t - 1 (capsules of local t at caps->caps[t * H ...]);
+// output dyn_mid[t][s][y][x], signed 2-D partial squared distances.  run_rows:
+// the rows of the capsules' boxes, summed, at most over t; dyn_xy_words: the
+// shared memory words of a CTA.
+size_t dyn_xy_words(int ny, int run_rows);
 cudaError_t launch_dyn_xy(const CapBatch *caps, const SlabMap *map, int H, int nx, int ny, int zlo, int S, int t0,
-                          int n_t, int cap,
-                          int32_t *dyn_mid, cudaStream_t stream);
+                          int n_t, int run_rows, int32_t *dyn_mid, cudaStream_t stream);
 
 // colmax[y][x] = largest value of the column (x, y) of sq [nz][ny][nx].
 cudaError_t launch_colmax(const int32_t *sq, int nx, int ny, int nz, int32_t *colmax, cudaStream_t stream);

@@ -207,9 +207,7 @@ int plan_composite(const pcdf_grid *grid, int T, int H, const int32_t *caps, Com
             return rc;
     p.S = p.zhi >= p.zlo ? p.zhi - p.zlo + 1 : 0;
     p.slab = (long long)T * p.S * grid->nx * grid->ny;
-    // stack bound of the analytic kernel: rows holding a run (<= sum of the
-    // capsules' y extents) plus two free rows per run (one run per capsule)
-    int ext_max = 0;
+    // rows of the capsules' boxes, at most over t
     for (int t = 0; t < T; ++t) {
         int ext = 0;
         for (int h = 0; h < H; ++h) {
@@ -217,10 +215,14 @@ int plan_composite(const pcdf_grid *grid, int T, int H, const int32_t *caps, Com
             if (c.lo[0] <= c.hi[0])
                 ext += c.hi[1] - c.lo[1] + 1;
         }
-        ext_max = std::max(ext_max, ext);
+        p.run_rows = std::max(p.run_rows, ext);
     }
-    p.cap = std::min(ext_max + 2 * H + 2, grid->ny + 2);
-    p.fused = H <= pcdf::kMaxCapsPerLaunch && pcdf::dyn_xy_fits(grid->ny, H, p.cap);
+    // beyond this bound on the capsules' rows the generic row and y passes
+    // run instead, and batches refuse the environment
+    const size_t cap = (size_t)std::min(p.run_rows + 2 * H + 2, grid->ny + 2);
+    p.fused = ((size_t)grid->ny * (H + 1) + cap * 128) * 4 <= 200 * 1024 &&
+              pcdf::dyn_xy_words(grid->ny, p.run_rows) * 4 <= 227 * 1024;
+    p.cap = (int)cap;
     plan_slab_map(T, H, p);
     if (p.S == 0)
         p.need = 0;
@@ -270,7 +272,7 @@ int composite_prepare(const pcdf_grid *grid, int T, int H, const CompositePlan &
             batch.count = nt * H;
             std::memcpy(batch.caps, p.ci.data() + (size_t)t0 * H, sizeof(pcdf::CapInfo) * nt * H);
             cudaError_t e =
-                pcdf::launch_dyn_xy(&batch, &map, H, grid->nx, grid->ny, p.zlo, p.S, t0, nt, p.cap, mid, st);
+                pcdf::launch_dyn_xy(&batch, &map, H, grid->nx, grid->ny, p.zlo, p.S, t0, nt, p.run_rows, mid, st);
             if (e != cudaSuccess)
                 return cuda_fail(e, "dynamic x+y pass");
         }

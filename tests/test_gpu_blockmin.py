@@ -67,3 +67,22 @@ def test_sparse_and_thick(shape):
     check(occ, oracle.edt(occ))
     occ[:, : shape[1] // 2] = 1
     check(occ, oracle.edt(occ))
+
+
+# capsule slices (the same search behind runs instead of row words): runs over
+# several words, to both walls, over whole rows and slices, overlapping humans,
+# rows that end inside a word, far columns
+@pytest.mark.parametrize("nx,ny,nz", [(65, 23, 17), (97, 40, 33), (200, 9, 21), (31, 64, 9), (400, 30, 12)])
+def test_capsule_slices(nx, ny, nz):
+    c = 16 * np.array([nx, ny, nz])
+    caps = [[[8, c[1] // 2, c[2] // 2, c[0] - 8, c[1] // 2, c[2] // 2, 40], [0, 0, 0, 0, 0, 0, 200]],   # wall to wall, and a corner
+            [[c[0] // 2, c[1] // 2, 0, c[0] // 2, c[1] // 2, c[2], 130], [c[0] // 2 + 60, c[1] // 2 + 30, 40, c[0] // 2 + 60, c[1] // 2 + 30, 90, 130]],
+            [[-200, c[1] // 2, c[2] // 2, 700, c[1] // 2, c[2] // 2, 16 * max(ny, nz)], [30, 30, 30, 30, 30, 30, 17]],   # whole slices
+            [[c[0] - 20, 20, 20, c[0] - 20, 20, 20, 30], [-900, -900, -900, -900, -900, -900, 10]]]                     # one small, one outside
+    caps = np.array(caps, np.int32)
+    static = oracle.edt(scenes.random_occupancy((nz, ny, nx), 0.002, np.random.default_rng(nx)))
+    grid = scenes.Grid(nx, ny, nz, 0.05)
+    sq, sdf = pcdf.build_predicted_composite(torch.from_numpy(static).to("cuda"), grid, caps)
+    want = oracle.predicted_composite(static, caps)
+    assert np.array_equal(sq.cpu().numpy(), want)
+    assert np.array_equal(sdf.cpu().numpy().view(np.int32), oracle.sdf_from_sq(want, 0.05).view(np.int32))
