@@ -197,11 +197,9 @@ int pcdf_composite_slab(const pcdf_grid *grid, int32_t T, int32_t H, const int32
  * overlap or time them separately (same arguments and workspace; the
  * workspace carries the dynamic intermediate from the first to the second):
  *   prepare: the capsule row pass and y pass over the z-slab the capsules touch;
- *   finish:  the static column maxima, then the fused z pass, composite min
- *            and float epilogue for every t (where a column's largest static
- *            value is no larger than the humans' least 2-D partial, or a z lies
- *            far enough from the slab, the output is the static field without
- *            evaluating the humans' envelope). */
+ *   finish:  the fused z pass, composite min and float epilogue for every t
+ *            (blocks that no human can come nearer to than the static map are
+ *            copies of the static field). */
 int pcdf_composite_prepare(const pcdf_grid *grid, int32_t T, int32_t H, const int32_t *caps, void *workspace,
                            size_t workspace_bytes, void *stream);
 int pcdf_composite_finish(const pcdf_grid *grid, const int32_t *static_sq, const float *static_sdf, int32_t T,
@@ -211,8 +209,7 @@ int pcdf_composite_finish(const pcdf_grid *grid, const int32_t *static_sq, const
 /* The finish stage for the fields t = t0 .. t0 + nt - 1 only (0 <= t0,
  * nt >= 1, t0 + nt <= T): the outputs are the same [T][nz][ny][nx] arrays,
  * indexed by the absolute t, and only the range's fields are written.  A
- * caller can copy finished fields to the host while later ones are computed
- * (each call also recomputes the static column maxima). */
+ * caller can copy finished fields to the host while later ones are computed. */
 int pcdf_composite_finish_range(const pcdf_grid *grid, const int32_t *static_sq, const float *static_sdf, int32_t T,
                                 int32_t H, const int32_t *caps, int32_t t0, int32_t nt, int32_t *comp_sq,
                                 float *comp_sdf, void *workspace, size_t workspace_bytes, void *stream);

@@ -26,8 +26,9 @@
 //  * Of a candidate block only the elements are taken that the next one
 //    towards the output block does not beat in every column (a slice that
 //    repeats its neighbour's distances, as along the sides of a box, never
-//    counts): a byte per block and side, found when the tile is filled.  The
-//    same holds inside the block itself.
+//    counts): a byte per block and side, found when the tile is filled, the
+//    neighbouring block's nearest element included.  A block without such
+//    elements is no candidate.  The same holds inside the block itself.
 // On the 256^3 map of 60 boxes that leaves 3 to 7 elements per block of 8, on
 // one with 0.2 % of speckle 9 to 16.  Sums stay below 2^16 within 22 blocks;
 // beyond them the squared gap alone is kFar16, so a block whose results are
@@ -56,6 +57,7 @@ constexpr int kSqMin = -kBlk * kReach;        // squares for elements kSqMin .. 
 constexpr int kSqMax = kBlk * kReach + kBlk - 1;
 constexpr int kSqWords = kBlk * (kSqMax - kSqMin + 1);
 constexpr int kMaxBlocks = 512 / kBlk;        // PCDF_MAX_DIM
+constexpr int kNoCandidate = 1 << 29;         // bound of a block that cannot matter
 constexpr int kCap32 = 1 << 28;               // "no site" in the 32-bit search: sums stay below 2^31
 static_assert(kBlk * (kReach + 1) - (kBlk - 1) >= kFarDist, "blocks beyond the reach cannot improve a value below kFar16");
 static_assert(kFar16 + (kBlk * kReach + kBlk - 1) * (kBlk * kReach + kBlk - 1) < 65536 && kFar16 < 32768, "16-bit sums");
@@ -67,7 +69,7 @@ __host__ __device__ constexpr int blocks_of(int n) { return (n + kBlk - 1) / kBl
 // Shared words of a tile of n elements.
 __host__ __device__ constexpr size_t tile_words(int n)
 {
-    return kSqWords + kTileCols + 2 * kMaxBlocks + (size_t)blocks_of(n) * (kPitch * kBlk + 32);
+    return kSqWords + 2 * kMaxBlocks + (size_t)blocks_of(n) * (kPitch * kBlk + 32);
 }
 
 // two signed values as 16 bits each, clamped at +-kFar16 (low half: a)
@@ -92,13 +94,19 @@ struct Info {
     uint2 w;
     __device__ __forceinline__ uint32_t use(bool before) const { return (before ? w.x >> 8 : w.x) & 0xffu; }
     __device__ __forceinline__ uint32_t own() const { return (w.x >> 16) & 0xffu; }
+    // the least O or F of a block that counts, after or before another one
+    template <bool kF>
+    __device__ __forceinline__ int least16(bool after) const
+    {
+        return kF ? (int)(w.y >> 16) : (use(after) ? (int)(w.y & 0xffffu) : kNoCandidate);
+    }
     __device__ __forceinline__ bool occupied() const { return (w.x >> 24) & 1u; }
+    __device__ __forceinline__ bool flat() const { return (w.x >> 27) & 1u; }  // recorded as flat
     __device__ __forceinline__ bool without(bool f) const { return (w.x >> (f ? 26 : 25)) & 1u; }  // no site of O / F
 };
 
 struct Tile {
     uint32_t *sq;      // sq[8 (d - kSqMin) + j] = (d - j)^2 in both halves
-    int32_t *top;      // [64] column maxima
     uint2 *info;       // [nb]
     uint32_t *v;       // [8 nb][kPitch] packed values (lane l: word l), the largest value past the end
     uint32_t *lo;      // [nb][32] least O of each block in the lane's columns
@@ -106,10 +114,14 @@ struct Tile {
     __device__ __forceinline__ Tile(uint32_t *smem, int n_) : n(n_), nb(blocks_of(n_))
     {
         sq = smem;
-        top = reinterpret_cast<int32_t *>(sq + kSqWords);
-        info = reinterpret_cast<uint2 *>(top + kTileCols);
+        info = reinterpret_cast<uint2 *>(sq + kSqWords);
         v = reinterpret_cast<uint32_t *>(info + kMaxBlocks);
         lo = v + nb * kPitch * kBlk;
+    }
+    // a tile without squares, its parts anywhere
+    __device__ __forceinline__ Tile(uint2 *info_, uint32_t *v_, uint32_t *lo_, int n_, int nb_)
+        : sq(nullptr), info(info_), v(v_), lo(lo_), n(n_), nb(nb_)
+    {
     }
     // before the barrier that ends the stores
     __device__ __forceinline__ void init() const
@@ -119,8 +131,6 @@ struct Tile {
             reinterpret_cast<uint4 *>(sq)[i] =
                 make_uint4(both(d * d), both((d - 1) * (d - 1)), both((d - 2) * (d - 2)), both((d - 3) * (d - 3)));
         }
-        for (int i = threadIdx.x; i < kTileCols; i += blockDim.x)
-            top[i] = INT32_MIN;
     }
     __device__ __forceinline__ Info about(int b) const { return Info{info[b]}; }
     // One warp records block b, whose values are x.  without(f): the block
@@ -163,7 +173,38 @@ struct Tile {
         if (lane == 0 && PCDF_IN(b, kMaxBlocks))
             info[b] = make_uint2((bits & 0xffffu) | (((bits & 0x7fu) | ((bits >> 8) & 0xfeu)) << 16) | flags, wo | (wf << 16));
     }
+
+    // The same for a block of 8 elements that all are x, none of them past the end.
+    __device__ __forceinline__ void record_flat(int b, int lane, uint32_t x) const
+    {
+        const uint32_t o = part<false>(x), f = part<true>(x);
+        lo[b * 32 + lane] = o;
+        const bool occ = __any_sync(0xffffffffu, (x & 0x80008000u) != 0);
+        const uint32_t wo = __reduce_min_sync(0xffffffffu, min(o & 0xffffu, o >> 16));
+        const uint32_t wf = occ ? __reduce_min_sync(0xffffffffu, min(f & 0xffffu, f >> 16)) : 0u;
+        if (lane == 0 && PCDF_IN(b, kMaxBlocks))
+            info[b] = make_uint2(0x08000180u | (occ ? 1u << 24 : 0u), wo | (wf << 16));  // before: element 0, after: element 7
+    }
 };
+
+// One warp compares the last element of block b with the first of block b + 1
+// (after the barrier that ends the records; another one before the tile is
+// used): the one that the other beats in every column no longer counts beyond it.
+__device__ __forceinline__ void link(const Tile &t, int b, int lane)
+{
+    if (b + 1 >= t.nb)
+        return;
+    const uint32_t *p = t.v + (kBlk * (b + 1) - 1) * kPitch + lane;
+    const uint32_t here = part<false>(p[0]), there = part<false>(p[kPitch]), m = __vmaxu2(here, there);
+    const bool ge = __all_sync(0xffffffffu, m == here), le = __all_sync(0xffffffffu, m == there);
+    if (lane == 0) {  // bytes 0 and 1 of two blocks: no other warp writes them
+        uint8_t *q = reinterpret_cast<uint8_t *>(t.info + b);
+        if (ge)
+            q[0] &= 0x7fu;
+        if (le)
+            q[sizeof(uint2) + 1] &= 0xfeu;
+    }
+}
 
 // The elements of block b inside the column.
 __device__ __forceinline__ uint32_t in_column(const Tile &t, int b) { return (1u << min(t.n - kBlk * b, kBlk)) - 1u; }
@@ -172,9 +213,9 @@ __device__ __forceinline__ uint32_t in_column(const Tile &t, int b) { return (1u
 __device__ __forceinline__ int gap2(int m) { return (kBlk * m - kBlk + 1) * (kBlk * m - kBlk + 1); }
 
 // Calls go(s, gap2) for the candidate blocks b + s, |s| from c0 + 1 to c0 + 32
-// and at most kMost, in order of distance: lane i holds the bounds
-// key(least O or F, info) + gap2 of the two blocks c0 + 1 + i away, and only
-// those below um, which go may lower, are called for.
+// and at most kMost, in order of distance: lane i holds the bounds key(info,
+// whether the block lies after b) + gap2 of the two blocks c0 + 1 + i away,
+// and only those below um, which go may lower, are called for.
 template <bool kF, int kMost, class Key, class Go>
 __device__ __forceinline__ void outwards(const Tile &t, int b, int c0, int lane, int &um, const Key &key, const Go &go)
 {
@@ -182,9 +223,9 @@ __device__ __forceinline__ void outwards(const Tile &t, int b, int c0, int lane,
     int kl = INT32_MAX, kr = INT32_MAX;
     if (m <= kMost) {
         if (b - m >= 0)
-            kl = key(t.about(b - m)) + g;
+            kl = key(t.about(b - m), false) + g;
         if (b + m < t.nb)
-            kr = key(t.about(b + m)) + g;
+            kr = key(t.about(b + m), true) + g;
     }
     uint32_t rest = 0xffffffffu;
     for (;;) {
@@ -234,10 +275,11 @@ __device__ __forceinline__ void visit(uint32_t (&best)[kBlk], const uint32_t *sq
 }
 
 // The packed minima of block b over O or F and, in u, their maxima; returns
-// the largest of them in the warp (elements past the end and columns outside
-// the grid count as 0).
+// the largest of them in the warp.  Elements past the end count as 0, columns
+// outside the grid (alive: the lane's columns inside) not at all.
 template <bool kF>
-__device__ __forceinline__ int search16(uint32_t (&best)[kBlk], uint32_t &u, const Tile &t, int b, int lane, uint32_t own)
+__device__ __forceinline__ int search16(uint32_t (&best)[kBlk], uint32_t &u, const Tile &t, int b, int lane, uint32_t own,
+                                        uint32_t alive)
 {
     const uint32_t *src = t.v + kBlk * b * kPitch + lane;
 #pragma unroll
@@ -262,10 +304,10 @@ __device__ __forceinline__ int search16(uint32_t (&best)[kBlk], uint32_t &u, con
         for (int j = 0; j < kBlk; ++j)
             best[j] = kBlk * b + j < t.n ? best[j] : 0u;
     }
-    u = largest(best);
+    u = largest(best) & alive;
     int um = warp_largest(u);
     outwards<kF, kReach>(
-        t, b, 0, lane, um, [](const Info &i) { return (int)(kF ? i.w.y >> 16 : i.w.y & 0xffffu); },
+        t, b, 0, lane, um, [](const Info &i, bool after) { return i.least16<kF>(after); },
         [&](int s) {
             const int q = b + s;
             if (!kF) {
@@ -276,27 +318,26 @@ __device__ __forceinline__ int search16(uint32_t (&best)[kBlk], uint32_t &u, con
             if (!PCDF_IN(q, t.nb))
                 return;
             visit<kF>(best, t.sq, src, s, kF ? in_column(t, q) : t.about(q).use(s > 0));
-            u = largest(best);
+            u = largest(best) & alive;
             um = warp_largest(u);
         });
     return um;
 }
 
-// One warp computes block b: out.near(best, u) takes the lane's packed values of
-// a block of free voxels whose results are below kFar16 (u: their maxima),
-// out.any(row, r0, r1) any value.  False (warp-uniform, nothing written): some
+// One warp computes block b: out.near(row, best) takes the lane's packed values
+// of a block of free voxels whose results are below kFar16, out.any(row, r0, r1) any value.  False (warp-uniform, nothing written): some
 // result is out of the 16-bit range.
 template <class Out>
-__device__ __forceinline__ bool block16(const Tile &t, int b, int lane, Out &out)
+__device__ __forceinline__ bool block16(const Tile &t, int b, int lane, uint32_t alive, Out &out)
 {
     uint32_t best[kBlk], u;
     const Info info = t.about(b);
-    if (search16<false>(best, u, t, b, lane, info.own()) >= kFar16)
+    if (search16<false>(best, u, t, b, lane, info.own(), alive) >= kFar16)
         return false;
     const int r0 = kBlk * b;
     if (info.occupied()) {
         uint32_t f[kBlk], uf;
-        if (search16<true>(f, uf, t, b, lane, 0) >= kFar16)
+        if (search16<true>(f, uf, t, b, lane, 0, alive) >= kFar16)
             return false;
 #pragma unroll
         for (int j = 0; j < kBlk; ++j)
@@ -308,7 +349,7 @@ __device__ __forceinline__ bool block16(const Tile &t, int b, int lane, Out &out
             if (r0 + j < t.n)
                 out.any(r0 + j, (int)(int16_t)(best[j] & 0xffffu), (int)best[j] >> 16);
     } else {
-        out.near(r0, best, u);
+        out.near(r0, best);
     }
     return true;
 }
@@ -337,6 +378,7 @@ __device__ __forceinline__ int warp_largest32(const int (&p)[kBlk], const int (&
 // and was recorded as such: the same search on their squares.
 struct DistTile {
     const Tile &t;
+    uint32_t alive;  // the lane's columns inside the grid
     template <bool kF>
     __device__ __forceinline__ void search(int (&p)[kBlk], int (&q)[kBlk], int b, int lane) const
     {
@@ -351,8 +393,10 @@ struct DistTile {
             }
         };
 #pragma unroll
-        for (int j = 0; j < kBlk; ++j)
-            p[j] = q[j] = kBlk * b + j < t.n ? kCap32 : 0;
+        for (int j = 0; j < kBlk; ++j) {
+            p[j] = kBlk * b + j < t.n && (alive & 0xffffu) ? kCap32 : 0;
+            q[j] = kBlk * b + j < t.n && (alive >> 16) ? kCap32 : 0;
+        }
         const uint32_t in = in_column(t, b);
         uint32_t rows = kF ? in : t.about(b).own() & in;
         if (!kF) {  // each element is a candidate for itself
@@ -369,9 +413,9 @@ struct DistTile {
         for (int c0 = 0; c0 < t.nb; c0 += 32)
             outwards<kF, kMaxBlocks>(
                 t, b, c0, lane, um,
-                [](const Info &i) {
-                    const int d = (int)(kF ? i.w.y >> 16 : i.w.y & 0xffffu);
-                    return d * d;
+                [](const Info &i, bool after) {
+                    const int d = i.least16<kF>(after);
+                    return d == kNoCandidate ? d : d * d;
                 },
                 [&](int s) {
                     visit(s, kF ? in_column(t, b + s) : t.about(b + s).use(s > 0) & in_column(t, b + s));
@@ -386,12 +430,15 @@ template <class Src>
 struct RawTile {
     const Tile &t;
     const Src &src;
+    uint32_t alive;  // the lane's columns inside the grid
     template <bool kF>
     __device__ __forceinline__ void search(int (&p)[kBlk], int (&q)[kBlk], int b, int lane) const
     {
 #pragma unroll
-        for (int j = 0; j < kBlk; ++j)
-            p[j] = q[j] = kBlk * b + j < t.n ? kCap32 : 0;
+        for (int j = 0; j < kBlk; ++j) {
+            p[j] = kBlk * b + j < t.n && (alive & 0xffffu) ? kCap32 : 0;
+            q[j] = kBlk * b + j < t.n && (alive >> 16) ? kCap32 : 0;
+        }
         int um = kCap32;
         auto go = [&](int s) {
 #pragma unroll 2
@@ -410,7 +457,8 @@ struct RawTile {
         for (int c0 = 0; c0 < t.nb; c0 += 32)
             outwards<kF, kMaxBlocks>(
                 t, b, c0, lane, um,
-                [](const Info &i) { return i.without(kF) ? kCap32 : (int)(kF ? i.w.y >> 16 : i.w.y & 0xffffu); }, go);
+                [](const Info &i, bool) { return i.without(kF) ? kNoCandidate : (int)(kF ? i.w.y >> 16 : i.w.y & 0xffffu); },
+                go);
     }
 };
 

@@ -3,7 +3,6 @@
 #include <cuda_runtime.h>
 
 #include "composite.cuh"
-#include "edt_full.cuh"
 
 namespace pcdf {
 namespace {
@@ -28,29 +27,21 @@ __global__ void __launch_bounds__(256, 4)
                            dyn_mid + ((long long)t * S + s) * nx * ny, sm);
 }
 
-// CTAs are ordered t-fastest, so the T CTAs of one column block run together
-// and read the static column block from DRAM once; each of them prefetches
-// every nt-th plane of that block into L2 before its own work.
+// CTAs are ordered t-fastest: those of one column block run together and the
+// static block comes from DRAM once.  Three CTAs of 8 warps (80 registers).
+// 256^3, T = 20, 3 humans: 471 us for 2.82 GB of outputs and inputs, 88 % of
+// the measured copy bandwidth (558 us, and 15 us of column maxima, with an
+// envelope per column and thread); 161 x 115 x 83, T = 9: 46 us (88 us).
 template <bool kSq, bool kSdfOut, bool kStaticSdf>
-__global__ void __launch_bounds__(128, 8)
-    k_composite_z(const int32_t *__restrict__ static_sq, const float *__restrict__ static_sdf,
-                  const int32_t *__restrict__ colmax, const int32_t *__restrict__ dyn_mid,
-                  const __grid_constant__ SlabMap map, int nx, int ny, int nz, int zlo, int S, int t0, int nt,
-                  int32_t *__restrict__ comp_sq, float *__restrict__ comp_sdf, float vox, int vec)
+__global__ void __launch_bounds__(comp::kThreadsZ, 3)
+    k_composite_z(const comp::Composite<kSq, kSdfOut, kStaticSdf> c, const __grid_constant__ SlabMap map, int t0, int nt,
+                  int steps)
 {
-    extern __shared__ uint32_t smem[];
-    const int t = t0 + (int)(blockIdx.x % nt);
-    comp::composite_block_short<kSq, kSdfOut, kStaticSdf>(static_sq, static_sdf, colmax, dyn_mid,
-                                                          map.on ? map.rep + t * S : nullptr, nx, ny, nz, zlo, S, t,
-                                                          (long long)(blockIdx.x / nt) * blockDim.x, comp_sq, comp_sdf,
-                                                          vox, vec != 0, smem, (int)(blockIdx.x % nt),
-                                                          vec ? nt : 0);
-}
-
-__global__ void __launch_bounds__(128) k_colmax(const int32_t *__restrict__ sq, long long V2, int nz,
-                                                int32_t *__restrict__ colmax)
-{
-    comp::colmax_block(sq, V2, nz, colmax);
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int groups = (nt + steps - 1) / steps, g = (int)blockIdx.x % groups;
+    comp::Composite<kSq, kSdfOut, kStaticSdf> cc = c;
+    cc.rep = map.on ? map.rep : nullptr;
+    cc.run(t0 + g * steps, min(steps, nt - g * steps), (long long)(blockIdx.x / groups) * full::kTileCols, smem);
 }
 
 __global__ void k_broadcast_static(const int32_t *__restrict__ static_sq, long long V, int t0, int nt,
@@ -90,50 +81,35 @@ cudaError_t launch_dyn_xy(const CapBatch *caps, const SlabMap *map, int H, int n
 namespace {
 
 template <bool kSq, bool kSdfOut, bool kStaticSdf>
-cudaError_t launch_cz(int nblk, int nthr, size_t smem, const int32_t *static_sq, const float *static_sdf,
-                      const int32_t *colmax, const int32_t *dyn_mid, const SlabMap *map, int nx, int ny, int nz,
-                      int zlo, int S, int t0, int nt, int32_t *comp_sq, float *comp_sdf, float vox, int vec,
+cudaError_t launch_cz(const comp::Composite<kSq, kSdfOut, kStaticSdf> &c, const SlabMap *map, int t0, int nt,
                       cudaStream_t stream)
 {
     auto kern = k_composite_z<kSq, kSdfOut, kStaticSdf>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(kern);
     if (e != cudaSuccess)
         return e;
-    kern<<<(unsigned)nblk, nthr, smem, stream>>>(static_sq, static_sdf, colmax, dyn_mid, *map, nx, ny, nz, zlo, S,
-                                                 t0, nt, comp_sq, comp_sdf, vox, vec);
+    // three CTAs per SM share its shared memory
+    const int steps = comp::steps_per_cta(c.zlo, c.S, c.nz, nt, 72 * 1024);
+    const size_t smem = steps * comp::slab_words(c.zlo, c.S, c.nz) * sizeof(uint32_t);
+    const int ntile = (c.V2 + full::kTileCols - 1) / full::kTileCols;
+    kern<<<(unsigned)(ntile * ((nt + steps - 1) / steps)), comp::kThreadsZ, smem, stream>>>(c, *map, t0, nt, steps);
     return cudaGetLastError();
 }
-
-bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 }  // namespace
 
-cudaError_t launch_colmax(const int32_t *sq, int nx, int ny, int nz, int32_t *colmax, cudaStream_t stream)
+cudaError_t launch_composite_z(const int32_t *static_sq, const float *static_sdf, const int32_t *dyn_mid,
+                               const SlabMap *map, int nx, int ny, int nz, int zlo, int S, int t0, int nt,
+                               int32_t *comp_sq, float *comp_sdf, float vox, cudaStream_t stream)
 {
-    const long long V2 = (long long)nx * ny;
-    k_colmax<<<(unsigned)((V2 + 31) / 32), 128, 0, stream>>>(sq, V2, nz, colmax);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_composite_z(const int32_t *static_sq, const float *static_sdf, const int32_t *colmax,
-                               const int32_t *dyn_mid, const SlabMap *map, int nx, int ny, int nz, int zlo, int S,
-                               int t0, int nt, int32_t *comp_sq, float *comp_sdf, float vox, cudaStream_t stream)
-{
-    const long long V2 = (long long)nx * ny;
-    const int words = S + 2 + (S + 31) / 32;
-    int nthr = 128;
-    while (nthr > 32 && (size_t)nthr * words * sizeof(uint32_t) > 200 * 1024)
-        nthr >>= 1;
-    const size_t smem = (size_t)nthr * words * sizeof(uint32_t);
-    const int nblk = (int)((V2 + nthr - 1) / nthr * nt);
     const bool sq = comp_sq != nullptr, sd = comp_sdf != nullptr, st = static_sdf != nullptr && sd;
-    // 16-byte copies of all-static column blocks: every plane and column
-    // block starts on a 16-byte boundary
-    const int vec = V2 % 4 == 0 && aligned16(static_sq) && (!st || aligned16(static_sdf)) &&
-                    (!sq || aligned16(comp_sq)) && (!sd || aligned16(comp_sdf));
+    // two adjacent columns in 8 bytes: every row of every field starts on such a boundary
+    const bool vec = nx * ny % 2 == 0 && (((uintptr_t)static_sq | (uintptr_t)(st ? static_sdf : nullptr) |
+                                           (uintptr_t)comp_sq | (uintptr_t)comp_sdf | (uintptr_t)dyn_mid) & 7u) == 0;
 #define PCDF_CZ(a, b, c)                                                                                            \
-    return launch_cz<a, b, c>(nblk, nthr, smem, static_sq, static_sdf, colmax, dyn_mid, map, nx, ny, nz, zlo, S, t0, \
-                              nt, comp_sq, comp_sdf, vox, vec, stream)
+    return launch_cz<a, b, c>({static_sq, static_sdf, dyn_mid, nullptr, comp_sq, comp_sdf, nx * ny, nz, zlo, S, vox, \
+                               vec},                                                                               \
+                              map, t0, nt, stream)
     if (sq && sd && st)
         PCDF_CZ(true, true, true);
     if (sq && sd)

@@ -1,5 +1,5 @@
 // Predicted composite fields (Sec. 6 composition, Sec. 8 sequence of fields)
-// on sm_103a: device code shared by the stand-alone kernels and the batched
+// on sm_103a: device code shared by the stand-alone kernel and the batched
 // persistent kernel.
 //
 // The field of the humans at time t is the exact signed EDT of the voxels
@@ -11,507 +11,548 @@
 //                of the static EDT (capsule_xy_block in edt_full.cuh).
 //                Output: the 2-D partial field of the slice (signed int32),
 //                with no row-pass intermediate in memory.
-//  k_colmax     the largest static value of every column (x, y).
-//  k_composite_z thread per (column (x, y), t): the z envelope of the slab's
-//                2-D partials, evaluated at every z, min with the static
-//                field, float epilogue; the T CTAs that share a static column
-//                block run together so that block is read from DRAM once.
+//  k_composite_z one CTA per (64 columns, up to kMaxSteps time steps): the z
+//                pass over the slab fused with the min against the static
+//                field and the float epilogue.
 //
-// The humans' field of a column is never below gmin, the least 2-D partial of
-// its slab, and at z outside the slab it is at least gmin plus the squared
-// distance to the slab.  Where the column's largest static value does not
-// exceed that bound the composite is the static field: a column with
-// colmax <= gmin is a copy of the static column, a CTA of such columns copies
-// its block with 16-byte accesses, and other columns evaluate the envelope
-// only in the z window around the slab where the humans can be nearer.
+// The CTA keeps the slab's partials of its columns and steps in shared memory
+// as the tiles of blockmin.cuh (clamped to 16 bits, with the bounds of their
+// blocks of 8 slices).  A warp then takes blocks of 8 slices of the grid: it
+// loads the static block once and, for each t, starts from the static values
+// and lowers them by the slab elements that can matter: those whose block's
+// least partial plus squared gap lies below the block's largest value.  For
+// most blocks there is none and the static block is stored as it is; no
+// bounds of the static field are needed beforehand.  Where the humans are
+// nearer the float field is the root of the new value, elsewhere the static
+// float field itself.  Voxels inside a human take the distance to the free
+// voxels (set F), from the same tile.  A block left with a value past the
+// 16-bit range is done again in 32 bits from the partials.
+//
+// Bound by the stores: T fields of 8 bytes per voxel.
 #pragma once
 
-#include "edt_common.cuh"
-
-#ifndef PCDF_EMIT_CHUNK
-#define PCDF_EMIT_CHUNK 6  // static values loaded ahead per lane in the z loops
-#endif
+#include "blockmin.cuh"
+#include "edt_full.cuh"
 
 namespace pcdf {
 namespace comp {
 
+using namespace blockmin;
 
-// ---------------------------------------------------------------------------
-// k_composite_z
-// ---------------------------------------------------------------------------
-// Shared memory per thread, [slot][thread]: slots 1..S hold the staged slab
-// column (slab element e in slot e + 1); slot 0 and slot S + 1 give the
-// in-place stacks room for the sites just below and above the slab; then the
-// occupancy bits of the slab column.
-//
-// Set F (distance to free voxels, output at the voxels inside a human) runs
-// first, in place over the staged column, and writes its outputs directly;
-// the column is then reloaded and set O (distance to the humans, output
-// everywhere else) is built in place and walked along z.  Where the static
-// field is nearer than the humans the float output is the static float field
-// itself (same value, no square root).
+constexpr int kMaxSteps = 4;   // time steps per CTA: the static block is read once for all of them
+constexpr int kThreadsZ = 256;     // of k_composite_z; any whole number of warps from 4 on
+static_assert(kMaxSteps * (kMaxBlocks / 4) <= 64, "a warp's blocks and steps in one mask");
 
-// Output flags: which of the two fields are written, whether the static
-// float field is available.
+// The z blocks [first, first + count) that a slab's tile covers: its slices
+// and one on either side (free voxels next to an occupied one).
+struct SlabBlocks {
+    int first, count;
+};
+__host__ __device__ inline SlabBlocks slab_blocks(int zlo, int S, int nz)
+{
+    if (S <= 0)
+        return SlabBlocks{0, 0};
+    const int lo = zlo > 0 ? zlo - 1 : 0, hi = zlo + S < nz ? zlo + S : nz - 1;
+    return SlabBlocks{lo / kBlk, hi / kBlk - lo / kBlk + 1};
+}
+// Shared words of one step's tile.
+__host__ __device__ inline size_t slab_words(int zlo, int S, int nz)
+{
+    const size_t nb = (size_t)slab_blocks(zlo, S, nz).count;
+    return (nb * (2 + kPitch * kBlk + 32) + 3) / 4 * 4;
+}
+// Time steps that a CTA takes together within `limit` shared bytes.
+__host__ inline int steps_per_cta(int zlo, int S, int nz, int T, size_t limit)
+{
+    const size_t w = slab_words(zlo, S, nz) * 4;
+    int most = kMaxSteps;
+    while (most > 1 && most * w > limit)
+        --most;
+    const int groups = (T + most - 1) / most;
+    return (T + groups - 1) / groups;
+}
+
+// (d - j)^2 in both halves, 8 words for each offset d from kSqMin on: read
+// through L1, so that a CTA need not build it.
+struct alignas(16) SquareTable {
+    uint32_t w[kSqWords];
+};
+constexpr SquareTable square_table()
+{
+    SquareTable t{};
+    for (int d = kSqMin; d <= kSqMax; ++d)
+        for (int j = 0; j < kBlk; ++j)
+            t.w[kBlk * (d - kSqMin) + j] = both((d - j) * (d - j));
+    return t;
+}
+static __device__ const SquareTable g_squares = square_table();
+
 template <bool kSq, bool kSdfOut, bool kStaticSdf>
-struct Out {
-    int32_t *ocol;
-    float *fcol;
+struct Composite {
+    const int32_t *static_sq;
+    const float *static_sdf;
+    const int32_t *dyn_mid;  // [T][S][V2] slab partials
+    const uint8_t *rep;      // [T][S]: slab element e is stored in slice rep[t][e] (NULL: e)
+    int32_t *comp_sq;
+    float *comp_sdf;
+    int V2, nz, zlo, S;
     float vox;
-    __device__ __forceinline__ void put(int o, int32_t sv, float sf, int32_t d) const
+    bool vec;  // two adjacent columns per lane, moved in 8 bytes (else two 32 apart)
+
+    // Slab element of slice z (-1: outside the slab, no human there).
+    __device__ __forceinline__ int element(int z) const { return z >= zlo && z < zlo + S ? z - zlo : -1; }
+    __device__ __forceinline__ int stored(int t, int e) const { return rep ? rep[t * S + e] : e; }
+
+    // Partials of slab element e at time t in the lane's columns (dead: none).
+    template <bool kVec>
+    __device__ __forceinline__ void partial(int t, int e, int o, const bool (&live)[2], int &v0, int &v1) const
     {
-        const int32_t cv = min(sv, d);
-        if (kSq)
-            __stcs(ocol + o, cv);
-        if (kSdfOut) {
-            float f;
-            if (kStaticSdf && sv <= d)
-                f = sf;
-            else
-                f = sq_to_sdf_fast(cv, vox);
-            __stcs(fcol + o, f);
+        v0 = v1 = kInf32;
+        if (e < 0 || !live[0])
+            return;
+        const int slice = stored(t, e);
+        const int32_t *p = dyn_mid + ((long long)t * S + slice) * V2 + o;
+        if (!PCDF_IN(slice, S) || !PCDF_IN(o, V2))
+            return;
+        if (kVec) {
+            const int2 v = __ldcg(reinterpret_cast<const int2 *>(p));
+            v0 = v.x;
+            v1 = v.y;
+        } else {
+            v0 = __ldcg(p);
+            if (live[1] && PCDF_IN(o + 32, V2))
+                v1 = __ldcg(p + 32);
         }
     }
-};
 
-template <bool kCoherent, class T>
-__device__ __forceinline__ T ldx(const T *p)
-{
-    if (kCoherent)
-        return __ldcg(p);
-    return __ldg(p);
-}
-
-// Outputs for z in [z0, z1).  kEval: the humans' distance is the envelope O
-// where useO holds (else +INF: the static field); kCheck: skip the occupied
-// slab voxels where useMk holds (set F wrote them).  Lanes of a warp that
-// share the bounds keep the loads and stores of a z coalesced; offsets
-// z * V2 stay below 2^31.
-template <bool kCheck, bool kEval, bool kCoherent, class O_t>
-__device__ __forceinline__ void emit_range(int z0, int z1, EnvCursor &O, bool useO, const uint32_t *mk, bool useMk,
-                                           int zlo, int nthr, const int32_t *scol, const float *sfcol, int V2,
-                                           const O_t &out, int nz_chk = 1 << 30)
-{
-    constexpr bool kStaticSdf = O_t::kHaveStatic;
-    constexpr int kC = PCDF_EMIT_CHUNK;
-    int z = z0;
-    for (; z + kC <= z1; z += kC) {
-        int32_t sv[kC];
-        float sf[kC];
+    // The static block of 8 slices at offset i0: the first r0 rows of the
+    // lane's first column and the first r1 of its second (others: 0).
+    template <bool kVec>
+    __device__ __forceinline__ void load(int i0, int r0, int r1, int2 (&s)[kBlk], float2 (&f)[kBlk]) const
+    {
+        const int32_t *p = static_sq + i0;
+        const float *g = static_sdf + (kStaticSdf ? i0 : 0);
 #pragma unroll
-        for (int i = 0; i < kC; ++i) {
-            const bool ok = PCDF_IN(z + i, nz_chk);
-            sv[i] = ok ? ldx<kCoherent>(scol + (z + i) * V2) : kInf32;
-            if (kStaticSdf)
-                sf[i] = ok ? ldx<kCoherent>(sfcol + (z + i) * V2) : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < kC; ++i) {
-            const int zz = z + i;
-            if (kCheck && useMk) {
-                const int e = zz - zlo;
-                if ((mk[(e >> 5) * nthr] >> (e & 31)) & 1u)
-                    continue;
+        for (int k = 0; k < kBlk; ++k, p += V2, g += kStaticSdf ? V2 : 0) {
+            s[k] = make_int2(0, 0);
+            f[k] = make_float2(0.f, 0.f);
+            if (kVec) {
+                if (k < r0 && PCDF_IN(i0 + k * V2 + 1, V2 * nz)) {
+                    s[k] = __ldcg(reinterpret_cast<const int2 *>(p));
+                    if (kStaticSdf)
+                        f[k] = __ldcg(reinterpret_cast<const float2 *>(g));
+                }
+            } else {
+                if (k < r0 && PCDF_IN(i0 + k * V2, V2 * nz)) {
+                    s[k].x = __ldcg(p);
+                    if (kStaticSdf)
+                        f[k].x = __ldcg(g);
+                }
+                if (k < r1 && PCDF_IN(i0 + k * V2 + 32, V2 * nz)) {
+                    s[k].y = __ldcg(p + 32);
+                    if (kStaticSdf)
+                        f[k].y = __ldcg(g + 32);
+                }
             }
-            const int32_t d = (kEval && useO) ? O.eval(zz) : kInf32;
-            if (PCDF_IN(zz, nz_chk))
-                out.put(zz * V2, sv[i], kStaticSdf ? sf[i] : 0.f, d);
+        }
+        if (kSdfOut && !kStaticSdf) {
+#pragma unroll
+            for (int k = 0; k < kBlk; ++k)
+                f[k] = make_float2(sq_to_sdf_fast(s[k].x, vox), sq_to_sdf_fast(s[k].y, vox));
         }
     }
-    for (; z < z1; ++z) {
-        if (kCheck && useMk) {
-            const int e = z - zlo;
-            if ((mk[(e >> 5) * nthr] >> (e & 31)) & 1u)
-                continue;
-        }
-        const int32_t d = (kEval && useO) ? O.eval(z) : kInf32;
-        if (PCDF_IN(z, nz_chk))
-            out.put(z * V2, ldx<kCoherent>(scol + z * V2), kStaticSdf ? ldx<kCoherent>(sfcol + z * V2) : 0.f, d);
-    }
-}
 
-// Outputs of one column over [0, nz) with the column's own bounds: below
-// its occupied run, the run (skipping its voxels), above it; `empty`: set O
-// has no site.
-template <bool kCoherent, class O_t>
-__device__ __forceinline__ void emit_all(int za, int zb, int nz, bool empty, EnvCursor &O, const uint32_t *mk,
-                                         int zlo, int nthr, const int32_t *scol, const float *sfcol, int V2,
-                                         const O_t &out)
-{
-    if (empty) {
-        emit_range<false, false, kCoherent>(0, za, O, false, mk, false, zlo, nthr, scol, sfcol, V2, out);
-        emit_range<true, false, kCoherent>(za, zb, O, false, mk, true, zlo, nthr, scol, sfcol, V2, out);
-        emit_range<false, false, kCoherent>(zb, nz, O, false, mk, false, zlo, nthr, scol, sfcol, V2, out);
-    } else {
-        emit_range<false, true, kCoherent>(0, za, O, true, mk, false, zlo, nthr, scol, sfcol, V2, out);
-        emit_range<true, true, kCoherent>(za, zb, O, true, mk, true, zlo, nthr, scol, sfcol, V2, out);
-        emit_range<false, true, kCoherent>(zb, nz, O, true, mk, false, zlo, nthr, scol, sfcol, V2, out);
-    }
-}
-
-template <bool kSq, bool kSdfOut, bool kStaticSdf>
-struct OutT : Out<kSq, kSdfOut, kStaticSdf> {
-    static constexpr bool kHaveStatic = kStaticSdf;
-};
-
-// 4-byte asynchronous copy global -> shared (no register staging); the
-// thread's copies complete at cp_async_wait_all.
-__device__ __forceinline__ void cp_async4(void *smem_dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
-                 "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned, bytes a
-// multiple of 16); nothing waits for it.
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// Largest value of each column c of a field [nz][V2]: warp w of the CTA reads
-// the z quarter w of 32 consecutive columns (lane = column).
-__device__ __forceinline__ void colmax_block(const int32_t *__restrict__ sq, long long V2, int nz,
-                                             int32_t *__restrict__ colmax)
-{
-    __shared__ int32_t part[4][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long c = (long long)blockIdx.x * 32 + lane;
-    const int z0 = (int)((long long)nz * w / 4), z1 = (int)((long long)nz * (w + 1) / 4);
-    int32_t m = INT32_MIN;
-    if (c < V2) {
-        const int32_t *col = sq + c;
-#pragma unroll 8
-        for (int z = z0; z < z1; ++z)
-            if (PCDF_IN(z, nz))
-                m = max(m, __ldg(col + (long long)z * V2));
-    }
-    part[w][lane] = m;
-    __syncthreads();
-    if (w == 0 && c < V2 && PCDF_IN(c, V2))
-        colmax[c] = max(max(part[0][lane], part[1][lane]), max(part[2][lane], part[3][lane]));
-}
-
-// The static field as the composite of time t on planes [z0, z1) of columns
-// [col0, col0 + ncols) (ncols a multiple of 4): 16-byte loads and stores,
-// thread tid on the column quad tid % nq of the planes z0 + tid / nq,
-// z0 + tid / nq + nthr / nq, ...  Needs V2 % 4 == 0, col0 % 4 == 0 and 16-byte
-// aligned fields.
-template <bool kSq, bool kSdfOut, bool kStaticSdf, bool kCoherent>
-__device__ __forceinline__ void copy_static_planes(const int32_t *__restrict__ static_sq,
-                                                   const float *__restrict__ static_sdf, long long V2, int nz, int z0,
-                                                   int z1, long long col0, int ncols, int32_t *__restrict__ osq,
-                                                   float *__restrict__ osdf, float vox)
-{
-    const int nq = ncols >> 2;
-    const int zstep = blockDim.x / nq;
-    const int qd = threadIdx.x % nq, zfirst = threadIdx.x / nq;
-    if (zfirst >= zstep)
-        return;
-    const long long base = col0 + 4 * qd;
-#pragma unroll 4
-    for (int z = z0 + zfirst; z < z1; z += zstep) {
-        const long long o = (long long)z * V2 + base;
-        if (!PCDF_IN(o + 3, V2 * nz))
-            continue;
-        const int4 sv = ldx<kCoherent>(reinterpret_cast<const int4 *>(static_sq + o));
-        if (kSq)
-            __stcs(reinterpret_cast<int4 *>(osq + o), sv);
-        if (kSdfOut) {
-            float4 f;
-            if (kStaticSdf)
-                f = ldx<kCoherent>(reinterpret_cast<const float4 *>(static_sdf + o));
-            else
-                f = make_float4(sq_to_sdf_fast(sv.x, vox), sq_to_sdf_fast(sv.y, vox), sq_to_sdf_fast(sv.z, vox),
-                                sq_to_sdf_fast(sv.w, vox));
-            __stcs(reinterpret_cast<float4 *>(osdf + o), f);
-        }
-    }
-}
-
-// Sets F and O of the column staged in tile (slot e + 1 holds slab element
-// e).  occ: some slab voxel of the column may lie inside a human; then mk
-// receives the occupancy bits, set F is built in place over the staged
-// column, its outputs (the occupied voxels) are written and the column is
-// staged again.  Set O is then built in place.  Returns the top of the set O
-// stack (-1: no site); [za, zb) is the z range of the occupied voxels
-// ([nz, nz) if none).
-template <bool kCoherent, class O_t>
-__device__ __forceinline__ int build_sets(uint32_t *tile, uint32_t *mk, bool occ, int nthr, int S, int nz, int zlo,
-                                          const int32_t *scol, const float *sfcol, const int32_t *dcol, long long V2,
-                                          const O_t &out, int &za, int &zb, const uint8_t *rep = nullptr)
-{
-    constexpr bool kStaticSdf = O_t::kHaveStatic;
-    const int nw = (S + 31) >> 5;
-    const int V2i = (int)V2;
-    int firstOcc = S, lastOcc = -1;
-    if (occ) {
-        for (int w = 0; w < nw; ++w) {
-            uint32_t bits = 0;
-            const int e0 = w << 5, cnt = min(32, S - e0);
-            for (int b = 0; b < cnt; ++b)
-                bits |= (uint32_t)((int32_t)tile[(e0 + b + 1) * nthr] < 0) << b;
-            mk[w * nthr] = bits;
-            if (bits) {
-                if (firstOcc == S)
-                    firstOcc = e0 + __ffs(bits) - 1;
-                lastOcc = e0 + 31 - __clz(bits);
+    // A row of the output at offset i (in0, in1: whether the lane's columns take part).
+    template <bool kVec>
+    __device__ __forceinline__ void store(int32_t *q, float *g, int i, bool in0, bool in1, int2 s, float2 f) const
+    {
+        if (kVec) {
+            if (in0 && PCDF_IN(i + 1, V2 * nz)) {
+                if (kSq)
+                    __stcs(reinterpret_cast<int2 *>(q), s);
+                if (kSdfOut)
+                    __stcs(reinterpret_cast<float2 *>(g), f);
+            }
+        } else {
+            if (in0 && PCDF_IN(i, V2 * nz)) {
+                if (kSq)
+                    __stcs(q, s.x);
+                if (kSdfOut)
+                    __stcs(g, f.x);
+            }
+            if (in1 && PCDF_IN(i + 32, V2 * nz)) {
+                if (kSq)
+                    __stcs(q + 32, s.y);
+                if (kSdfOut)
+                    __stcs(g + 32, f.y);
             }
         }
     }
-    auto occupied = [&](int z) {
-        const int e = z - zlo;
-        return occ && e >= 0 && e < S && ((mk[(e >> 5) * nthr] >> (e & 31)) & 1u);
+
+    __device__ __forceinline__ Tile tile(uint32_t *smem, int step, const SlabBlocks &sb) const
+    {
+        uint32_t *w = smem + step * slab_words(zlo, S, nz);
+        uint32_t *v = w + (2 * sb.count + 3) / 4 * 4;
+        return Tile(reinterpret_cast<uint2 *>(w), v, v + sb.count * kPitch * kBlk, nz, sb.count);
+    }
+
+    // Bound of slab block q for block c (both counted from the tile's first).
+    template <bool kF>
+    __device__ __forceinline__ int bound(const Tile &t, int q, int c) const
+    {
+        const int m = abs(q - c);
+        const Info i = t.about(q);
+        return !kF && m == 0 ? (int)(i.w.y & 0xffffu) : i.template least16<kF>(q > c) + (m ? gap2(m) : 0);
+    }
+
+    // Can an element of the slab lie below um in block b?
+    __device__ __forceinline__ bool reached(const Tile &t, int first, int b, int lane, int um) const
+    {
+        bool any = false;
+        for (int q = lane; q < t.nb; q += 32)
+            any |= bound<false>(t, q, b - first) < um;
+        return __any_sync(0xffffffffu, any);
+    }
+
+    // Lowers best (the lane's packed values of block b) by the slab's O or F;
+    // u, um: their largest in the lane and the warp, kept up to date.
+    template <bool kF>
+    __device__ __forceinline__ void lower(uint32_t (&best)[kBlk], uint32_t &u, int &um, uint32_t alive, const Tile &t,
+                                          int first, int b, int lane) const
+    {
+        const int c = b - first;  // the block itself, maybe outside the tile
+        const uint32_t *src = t.v + kBlk * c * kPitch + lane;
+        for (int q0 = 0; q0 < t.nb; q0 += 32) {
+            const int key = q0 + lane < t.nb ? bound<kF>(t, q0 + lane, c) : INT32_MAX;
+            const uint32_t upto = 0xffffffffu >> (31 - min(max(c - q0, 0), 31));
+            uint32_t rest = 0xffffffffu;
+            for (;;) {
+                const uint32_t a = __ballot_sync(0xffffffffu, key < um) & rest;
+                if (!a)
+                    break;
+                const int below = 31 - __clz(a & upto), above = __ffs(a & ~upto) - 1;  // -1: none
+                const int i = above < 0 || (below >= 0 && c - q0 - below <= above - (c - q0)) ? below : above;
+                rest &= ~(1u << i);
+                const int Q = q0 + i, s = Q - c;
+                if (!kF && s != 0) {
+                    const int gap = gap2(abs(s));
+                    if (!__any_sync(0xffffffffu, __viaddmin_u16x2(t.lo[Q * 32 + lane], both(gap), u) != u))
+                        continue;
+                }
+                uint32_t rows;
+                if (kF && t.about(Q).flat()) {  // the nearest slice stands for all
+                    rows = s ? (s > 0 ? 0x01u : 0x80u) : 0u;
+                    if (s == 0) {
+#pragma unroll
+                        for (int k = 0; k < kBlk; ++k)
+                            best[k] = __vminu2(best[k], part<true>(src[k * kPitch]));
+                    }
+                } else if (kF) {
+                    rows = (1u << min(nz - kBlk * (first + Q), kBlk)) - 1u;
+                } else if (s) {
+                    rows = t.about(Q).use(s > 0);
+                } else {  // each slice for itself, then those that count for others of the block
+#pragma unroll
+                    for (int k = 0; k < kBlk; ++k)
+                        best[k] = __vminu2(best[k], part<false>(src[k * kPitch]));
+                    rows = t.about(Q).own();
+                }
+                visit<kF>(best, g_squares.w, src, s, rows);
+                u = largest(best) & alive;
+                um = warp_largest(u);
+            }
+        }
+    }
+
+    // The value and its float at a voxel: static s (float f), the humans' d
+    // (positive: least of the static value and the distance, or anything
+    // larger; negative: inside a human).
+    __device__ __forceinline__ void pick(int s, float f, int d, int &cs, float &cf) const
+    {
+        cs = min(s, d);
+        cf = s <= d ? f : sq_to_sdf_fast(d, vox);
+    }
+
+    // Block b in the lane's columns: offset of its first row, rows of each column.
+    template <bool kVec>
+    struct Block {
+        int at, r0, r1;
+        __device__ __forceinline__ Block(const Composite &c, int b, int o, const bool (&live)[2])
+            : at(o + kBlk * b * c.V2), r0(live[0] ? min(c.nz - kBlk * b, kBlk) : 0), r1(live[1] ? min(c.nz - kBlk * b, kBlk) : 0)
+        {
+        }
+        __device__ __forceinline__ int32_t *sq_of(const Composite &c, int t) const
+        {
+            return kSq ? c.comp_sq + ((long long)t * c.V2 * c.nz + at) : nullptr;
+        }
+        __device__ __forceinline__ float *sdf_of(const Composite &c, int t) const
+        {
+            return kSdfOut ? c.comp_sdf + ((long long)t * c.V2 * c.nz + at) : nullptr;
+        }
     };
 
-    const int zo0 = zlo + firstOcc, zo1 = zlo + lastOcc;
-    if (lastOcc >= 0) {
-        // set F over [zo0 - 1, zo1 + 1]; free voxels are sites only next to an
-        // occupied one.  Site z sits in slot z - zlo + 1, read before written.
-        const int zr0 = max(zo0 - 1, 0), zr1 = min(zo1 + 1, nz - 1);
-        EnvBuilder B(tile + (zr0 - zlo + 1) * nthr, nthr, S + 2 - (zr0 - zlo + 1));
-        for (int z = zr0; z <= zr1; ++z) {
-            int g;
-            if (occupied(z)) {
-                const int32_t v = (int32_t)tile[(z - zlo + 1) * nthr];
-                if (v == -kInf32)
+    // best: the least of the static values s (negative ones as 0) and the
+    // distance to the humans; returns the warp's largest.
+    __device__ __forceinline__ int least_of(const Tile &tl, int first, int b, int lane, uint32_t alive, const int2 (&s)[kBlk],
+                                            uint32_t (&best)[kBlk]) const
+    {
+#pragma unroll
+        for (int k = 0; k < kBlk; ++k)
+            best[k] = part<false>(clamp16(s[k].x, s[k].y));
+        uint32_t u = largest(best) & alive;
+        int um = warp_largest(u);
+        lower<false>(best, u, um, alive, tl, first, b, lane);
+        return um;
+    }
+
+    // The CTA (4 warps or more) computes columns col0 .. col0 + 63 of time
+    // steps t0 .. t0 + nt - 1; smem: nt * slab_words().
+    __device__ __forceinline__ void run(int t0, int nt, long long col0, uint32_t *smem) const
+    {
+        if (vec)
+            run_as<true>(t0, nt, (int)col0, smem);
+        else
+            run_as<false>(t0, nt, (int)col0, smem);
+    }
+
+    // The tiles of the steps: values, bounds, links.
+    template <bool kVec>
+    __device__ __forceinline__ void fill(int t0, int nt, int o, const bool (&live)[2], const SlabBlocks &sb,
+                                         uint32_t *smem) const
+    {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        for (int Q = wid; Q < sb.count; Q += nw) {
+            const int e0 = kBlk * (sb.first + Q) - zlo;  // slab element of the block's first slice
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step) {
+                const int t = t0 + step;
+                const Tile tl = tile(smem, step, sb);
+                uint32_t *dst = tl.v + Q * kBlk * kPitch + lane;
+                const int32_t *src = dyn_mid + ((long long)t * S * V2 + o);
+                // lane k: where slice k of the block is stored (-1: outside the slab)
+                const int e = e0 + (lane & 7);
+                int slot = -1;
+                if (e >= 0 && e < S)
+                    slot = rep && PCDF_IN(e, S) ? rep[t * S + e] : e;
+                const int first = __shfl_sync(0xffffffffu, slot, 0);
+                auto get = [&](int at, int &v0, int &v1) {
+                    v0 = v1 = kInf32;
+                    if (at < 0 || !live[0] || !PCDF_IN(at, S) || !PCDF_IN(o, V2))
+                        return;
+                    const int32_t *p = src + at * V2;  // a slab holds less than 2^31 values
+                    if (kVec) {
+                        const int2 v = __ldcg(reinterpret_cast<const int2 *>(p));
+                        v0 = v.x;
+                        v1 = v.y;
+                    } else {
+                        v0 = __ldcg(p);
+                        if (live[1] && PCDF_IN(o + 32, V2))
+                            v1 = __ldcg(p + 32);
+                    }
+                };
+                // slices of equal cross-sections throughout (an upright human
+                // between its ends): one load, and all is known
+                if (__all_sync(0xffffffffu, slot == first) && first >= 0) {
+                    int a0, a1;
+                    get(first, a0, a1);
+                    const uint32_t v = clamp16(a0, a1);
+#pragma unroll
+                    for (int k = 0; k < kBlk; ++k)
+                        dst[k * kPitch] = v;
+                    tl.record_flat(Q, lane, v);
                     continue;
-                g = -v;
-            } else {
-                if (!occupied(z - 1) && !occupied(z + 1))
-                    continue;
-                g = 0;
+                }
+                int a0[kBlk], a1[kBlk];
+#pragma unroll
+                for (int k = 0; k < kBlk; ++k)
+                    get(__shfl_sync(0xffffffffu, slot, k), a0[k], a1[k]);
+                uint32_t v[kBlk], sign = 0;
+#pragma unroll
+                for (int k = 0; k < kBlk; ++k) {
+                    v[k] = clamp16(a0[k], a1[k]);
+                    sign |= v[k];
+                    dst[k * kPitch] = v[k];
+                }
+                tl.record(Q, lane, v, __any_sync(0xffffffffu, (sign & 0x80008000u) != 0), kFar16, [](bool) { return false; });
             }
-            B.push(z, g);
         }
-        EnvCursor F(tile + (zr0 - zlo + 1) * nthr, nthr, B.top);
-        for (int z = zo0; z <= zo1; ++z) {
-            if (!occupied(z))
+        __syncthreads();
+        for (int Q = wid; Q + 1 < sb.count; Q += nw)
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step)
+                link(tile(smem, step, sb), Q, lane);
+        __syncthreads();
+    }
+
+    template <bool kVec>
+    __device__ __forceinline__ void run_as(int t0, int nt, int col0, uint32_t *smem) const
+    {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        const SlabBlocks sb = slab_blocks(zlo, S, nz);
+        const int o = col0 + (kVec ? 2 * lane : lane);
+        const bool live[2] = {o < V2, o + (kVec ? 1 : 32) < V2};
+        const uint32_t alive = (live[0] ? 0x0000ffffu : 0u) | (live[1] ? 0xffff0000u : 0u);
+        fill<kVec>(t0, nt, o, live, sb, smem);
+
+        // Three loops over the warp's blocks and steps, from the lean to the
+        // rare: copies of the static block, blocks that a human can change,
+        // blocks with voxels inside a human.  In one loop the compiler's code
+        // for the rare paths slowed the others (366 M instead of 214 M
+        // instructions at 256^3, T = 20).
+        unsigned long long near = 0, inside = 0, far = 0;  // bit kMaxSteps * block + step
+        for (int b = wid, i = 0; kBlk * b < nz; b += nw, i += kMaxSteps) {
+            const Block<kVec> B(*this, b, o, live);
+            int2 s[kBlk];
+            float2 f[kBlk];
+            load<kVec>(B.at, B.r0, B.r1, s, f);
+            uint32_t u = 0;
+#pragma unroll
+            for (int k = 0; k < kBlk; ++k)
+                u = __vmaxu2(u, part<false>(clamp16(s[k].x, s[k].y)));
+            const int um = warp_largest(u & alive);
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step) {
+                const Tile tl = tile(smem, step, sb);
+                if (reached(tl, sb.first, b, lane, um) || (um >= kFar16 && sb.count)) {
+                    const int c = b - sb.first;
+                    if (c >= 0 && c < sb.count && tl.about(c).occupied())
+                        inside |= 1ull << (i + step);
+                    else
+                        near |= 1ull << (i + step);
+                } else {
+                    int32_t *q = B.sq_of(*this, t0 + step);
+                    float *g = B.sdf_of(*this, t0 + step);
+#pragma unroll
+                    for (int k = 0; k < kBlk; ++k, q += kSq ? V2 : 0, g += kSdfOut ? V2 : 0)
+                        store<kVec>(q, g, B.at + k * V2, k < B.r0, k < B.r1, s[k], f[k]);
+                }
+            }
+        }
+        unsigned long long todo = near;
+        for (int b = wid, i = 0; todo; b += nw, i += kMaxSteps, todo >>= kMaxSteps) {
+            if (!(todo & ((1u << kMaxSteps) - 1u)))
                 continue;
-            const int f = F.eval(z);
-            const int o = z * V2i;
-            if (PCDF_IN(z, nz))
-                out.put(o, ldx<kCoherent>(scol + o), kStaticSdf ? ldx<kCoherent>(sfcol + o) : 0.f,
-                        f < 0 ? -kInf32 : -f);
+            const Block<kVec> B(*this, b, o, live);
+            int2 s[kBlk];
+            float2 f[kBlk];
+            load<kVec>(B.at, B.r0, B.r1, s, f);
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step) {
+                if (!((todo >> step) & 1u))
+                    continue;
+                uint32_t best[kBlk];
+                if (least_of(tile(smem, step, sb), sb.first, b, lane, alive, s, best) >= kFar16) {
+                    far |= 1ull << (i + step);
+                    continue;
+                }
+                int32_t *q = B.sq_of(*this, t0 + step);
+                float *g = B.sdf_of(*this, t0 + step);
+#pragma unroll
+                for (int k = 0; k < kBlk; ++k, q += kSq ? V2 : 0, g += kSdfOut ? V2 : 0) {
+                    // the static value where it is the least (or negative)
+                    const int b0 = (int)(best[k] & 0xffffu), b1 = (int)(best[k] >> 16);
+                    int2 cs = s[k];
+                    float2 cf = f[k];
+                    if (b0 < s[k].x) {
+                        cs.x = b0;
+                        cf.x = kSdfOut ? full::root_near(b0, vox) : 0.f;
+                    }
+                    if (b1 < s[k].y) {
+                        cs.y = b1;
+                        cf.y = kSdfOut ? full::root_near(b1, vox) : 0.f;
+                    }
+                    store<kVec>(q, g, B.at + k * V2, k < B.r0, k < B.r1, cs, cf);
+                }
+            }
         }
-        // restore the staged column for set O
-#pragma unroll 8
-        for (int e = 0; e < S; ++e)
-            if (PCDF_IN(rep ? rep[e] : e, S))
-                tile[(e + 1) * nthr] = (uint32_t)ldx<kCoherent>(dcol + (long long)(rep ? rep[e] : e) * V2);
-    }
-
-    // set O over the slab: sites are the free slab voxels with a finite
-    // partial and the ends of the occupied runs (zero distance)
-    EnvBuilder B(tile + nthr, nthr, S + 1);
-    for (int e = 0; e < S; ++e) {
-        const int32_t v = (int32_t)tile[(e + 1) * nthr];
-        int g;
-        if (v >= 0) {
-            if (v == kInf32)
+        todo = inside;
+        for (int b = wid, i = 0; todo; b += nw, i += kMaxSteps, todo >>= kMaxSteps) {
+            if (!(todo & ((1u << kMaxSteps) - 1u)))
                 continue;
-            g = v;
-        } else {
-            const int z = zlo + e;
-            if (occupied(z - 1) && occupied(z + 1))
+            const Block<kVec> B(*this, b, o, live);
+            int2 s[kBlk];
+            float2 f[kBlk];
+            load<kVec>(B.at, B.r0, B.r1, s, f);
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step) {
+                if (!((todo >> step) & 1u))
+                    continue;
+                const Tile tl = tile(smem, step, sb);
+                uint32_t best[kBlk], fr[kBlk], uf = both(kFar16);
+                const int um = least_of(tl, sb.first, b, lane, alive, s, best);
+                int umf = kFar16;
+#pragma unroll
+                for (int k = 0; k < kBlk; ++k)
+                    fr[k] = kBlk * b + k < nz ? both(kFar16) : 0u;
+                lower<true>(fr, uf, umf, alive, tl, sb.first, b, lane);
+                if (um >= kFar16 || umf >= kFar16) {
+                    far |= 1ull << (i + step);
+                    continue;
+                }
+                int32_t *q = B.sq_of(*this, t0 + step);
+                float *g = B.sdf_of(*this, t0 + step);
+#pragma unroll
+                for (int k = 0; k < kBlk; ++k, q += kSq ? V2 : 0, g += kSdfOut ? V2 : 0) {
+                    const int f0 = (int)(fr[k] & 0xffffu), f1 = (int)(fr[k] >> 16);
+                    int2 cs;
+                    float2 cf;
+                    pick(s[k].x, f[k].x, f0 ? -f0 : (s[k].x < 0 ? kInf32 : (int)(best[k] & 0xffffu)), cs.x, cf.x);
+                    pick(s[k].y, f[k].y, f1 ? -f1 : (s[k].y < 0 ? kInf32 : (int)(best[k] >> 16)), cs.y, cf.y);
+                    store<kVec>(q, g, B.at + k * V2, k < B.r0, k < B.r1, cs, cf);
+                }
+            }
+        }
+
+        // rare, and written for few registers: a search with arrays here slowed
+        // the loop above (356 M instead of 254 M instructions at 256^3, T = 20)
+        for (int b = wid; far; b += nw, far >>= kMaxSteps)
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step)
+                if ((far >> step) & 1u)
+#pragma unroll 1
+                    for (int k = 0; k < kBlk && kBlk * b + k < nz; ++k)
+                        whole_column<kVec>(t0 + step, kBlk * b + k, o, live);
+    }
+
+    // Slice z of time t in 32 bits: both sets over the whole slab.
+    template <bool kVec>
+    __device__ __forceinline__ void whole_column(int t, int z, int o, const bool (&live)[2]) const
+    {
+        int o0 = kCap32, o1 = kCap32, f0 = kCap32, f1 = kCap32;
+        const int zend = min(zlo + S, nz - 1);  // a slice beyond the slab holds free voxels only
+#pragma unroll 1
+        for (int w = max(zlo - 1, 0); w <= zend; ++w) {
+            int v0, v1;
+            partial<kVec>(t, element(w), o, live, v0, v1);
+            const int d = (z - w) * (z - w);
+            o0 = min(o0, d + min(max(v0, 0), kCap32));
+            o1 = min(o1, d + min(max(v1, 0), kCap32));
+            f0 = min(f0, d + min(max(-v0, 0), kCap32));
+            f1 = min(f1, d + min(max(-v1, 0), kCap32));
+        }
+        int v0, v1;
+        partial<kVec>(t, element(z), o, live, v0, v1);
+        const int d0 = v0 < 0 ? (f0 >= kCap32 ? -kInf32 : -f0) : (o0 >= kCap32 ? kInf32 : o0);
+        const int d1 = v1 < 0 ? (f1 >= kCap32 ? -kInf32 : -f1) : (o1 >= kCap32 ? kInf32 : o1);
+        const int i = o + z * V2;
+        const long long w = t * (long long)V2 * nz + i;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = h * (kVec ? 1 : 32), d = h ? d1 : d0;
+            if (!live[h] || !PCDF_IN(i + j, V2 * nz))
                 continue;
-            g = 0;
-        }
-        B.push(zlo + e, g);
-    }
-    za = lastOcc >= 0 ? zo0 : nz;
-    zb = lastOcc >= 0 ? zo1 + 1 : nz;
-    return B.top;
-}
-
-// The CTA computes columns [col0, col0 + blockDim.x) of time t, one column
-// per thread with the column's own z ranges (used inside the batched kernel;
-// no block-level synchronisation); smem holds
-// blockDim.x * (S + 2 + ceil(S / 32)) words.
-template <bool kSq, bool kSdfOut, bool kStaticSdf, bool kCoherent>
-__device__ __forceinline__ void composite_block(const int32_t *__restrict__ static_sq,
-                                                const float *__restrict__ static_sdf,
-                                                const int32_t *__restrict__ dyn_mid, int nx, int ny, int nz, int zlo,
-                                                int S, int t, long long col0, int32_t *__restrict__ comp_sq,
-                                                float *__restrict__ comp_sdf, float vox, uint32_t *smem,
-                                                const uint8_t *__restrict__ rep = nullptr)
-{
-    const int nthr = blockDim.x, tid = threadIdx.x;
-    const long long V2 = (long long)nx * ny;
-    const long long c = col0 + tid;
-    if (c >= V2)
-        return;
-    uint32_t *tile = smem + tid;                              // slot k at tile[k * nthr]
-    uint32_t *mk = smem + (size_t)(S + 2) * nthr + tid;       // word w at mk[w * nthr]
-    const int32_t *dcol = dyn_mid + (long long)t * S * V2 + c;
-
-#pragma unroll 8
-    for (int e = 0; e < S; ++e) {
-        const int32_t *src = dcol + (long long)(rep ? rep[e] : e) * V2;
-        tile[(e + 1) * nthr] = (uint32_t)(kCoherent ? __ldcg(src) : __ldcs(src));
-    }
-
-    const long long V = V2 * nz;
-    const int32_t *scol = static_sq + c;
-    const float *sfcol = kStaticSdf ? static_sdf + c : nullptr;
-    OutT<kSq, kSdfOut, kStaticSdf> out;
-    out.ocol = kSq ? comp_sq + (long long)t * V + c : nullptr;
-    out.fcol = kSdfOut ? comp_sdf + (long long)t * V + c : nullptr;
-    out.vox = vox;
-    int za, zb;
-    const int top = build_sets<kCoherent>(tile, mk, true, nthr, S, nz, zlo, scol, sfcol, dcol, V2, out, za, zb, rep);
-    EnvCursor O(tile + nthr, nthr, top);
-    emit_all<kCoherent>(za, zb, nz, top < 0, O, mk, zlo, nthr, scol, sfcol, (int)V2, out);
-}
-
-// The CTA of k_composite_z: columns [col0, col0 + blockDim.x) of time t with
-// the static shortcuts.  colmax: the largest static value of every column;
-// rep (nullable: the identity): slab element e of time t is stored in slice
-// rep[e] (slices of equal capsule cross-sections computed once); vec: the
-// CTA may copy with 16-byte accesses.  pf_parts > 0 (needs vec): the CTA
-// first asks L2 to prefetch planes pf_part, pf_part + pf_parts, ... of its
-// static column block (bulk prefetches, no registers held), so that the
-// CTAs that share the block (one per t) split the block between them and
-// their loads of it hit L2.  Block-wide barriers: every thread of the CTA
-// calls.
-//  * every column static (colmax <= gmin): the CTA copies the static block;
-//  * else each column with dynamic influence has a window [w0, w1) (the slab
-//    and every z less than R slices from it, R the least integer with
-//    gmin + R^2 >= colmax; beyond it the static field wins).  Outside the
-//    union of the windows the block is copied (16-byte accesses when vec,
-//    else per column); inside it every lane of a warp runs the same z loops,
-//    so the accesses of a z stay coalesced, with the envelope (+INF for the
-//    static columns).
-template <bool kSq, bool kSdfOut, bool kStaticSdf>
-__device__ __forceinline__ void composite_block_short(const int32_t *__restrict__ static_sq,
-                                                      const float *__restrict__ static_sdf,
-                                                      const int32_t *__restrict__ colmax,
-                                                      const int32_t *__restrict__ dyn_mid,
-                                                      const uint8_t *__restrict__ rep, int nx, int ny, int nz,
-                                                      int zlo, int S, int t, long long col0,
-                                                      int32_t *__restrict__ comp_sq, float *__restrict__ comp_sdf,
-                                                      float vox, bool vec, uint32_t *smem, int pf_part = 0,
-                                                      int pf_parts = 0)
-{
-    __shared__ int s_w0, s_w1, s_occ;
-    const int nthr = blockDim.x, tid = threadIdx.x;
-    const long long V2 = (long long)nx * ny;
-    const long long c = col0 + tid;
-    const bool live = c < V2;
-    if (pf_parts > 0) {
-        // the block's columns of one plane: a multiple of 16 bytes from a
-        // 16-byte boundary (V2 % 4 == 0, col0 % 4 == 0, aligned fields)
-        const uint32_t nb = (uint32_t)min((long long)nthr, V2 - col0) * 4u;
-        for (int z = pf_part + pf_parts * tid; z < nz; z += pf_parts * nthr) {
-            const long long o = (long long)z * V2 + col0;
-            if (!PCDF_IN(o + nb / 4 - 1, V2 * nz))
-                continue;
-            prefetch_l2(static_sq + o, nb);
-            if (kStaticSdf)
-                prefetch_l2(static_sdf + o, nb);
+            const int s = static_sq[i + j];
+            const float f = kStaticSdf ? static_sdf[i + j] : (kSdfOut ? sq_to_sdf_fast(s, vox) : 0.f);
+            int cs;
+            float cf;
+            pick(s, f, d, cs, cf);
+            if (kSq)
+                comp_sq[w + j] = cs;
+            if (kSdfOut)
+                comp_sdf[w + j] = cf;
         }
     }
-    uint32_t *tile = smem + tid;                              // slot k at tile[k * nthr]
-    uint32_t *mk = smem + (size_t)(S + 2) * nthr + tid;       // word w at mk[w * nthr]
-    const int32_t *dcol = dyn_mid + (long long)t * S * V2 + c;
-    const long long V = V2 * nz;
-    if (tid == 0) {
-        s_w0 = nz;
-        s_w1 = 0;
-        s_occ = 0;
-    }
-
-    // stage the slab column with every load in flight at once
-    int32_t gmin = kInf32;
-    const int32_t cmax = live && PCDF_IN(c, V2) ? __ldg(colmax + c) : kInf32;
-    if (live) {
-        for (int e = 0; e < S; ++e)
-            if (PCDF_IN(rep ? rep[e] : e, S))
-                cp_async4(tile + (e + 1) * nthr, dcol + (long long)(rep ? rep[e] : e) * V2);
-        cp_async_wait_all();
-#pragma unroll 8
-        for (int e = 0; e < S; ++e)
-            gmin = min(gmin, (int32_t)tile[(e + 1) * nthr]);
-    }
-    // the humans' field of the column is >= gmin everywhere
-    const bool col_static = cmax <= gmin;
-    const int32_t *scol = static_sq + c;
-    const float *sfcol = kStaticSdf ? static_sdf + c : nullptr;
-    OutT<kSq, kSdfOut, kStaticSdf> out;
-    out.ocol = kSq ? comp_sq + (long long)t * V + c : nullptr;
-    out.fcol = kSdfOut ? comp_sdf + (long long)t * V + c : nullptr;
-    out.vox = vox;
-    const int V2i = (int)V2;
-    if (__syncthreads_and(!live || col_static)) {
-        if (vec) {
-            copy_static_planes<kSq, kSdfOut, kStaticSdf, false>(
-                static_sq, static_sdf, V2, nz, 0, nz, col0, (int)min((long long)nthr, V2 - col0),
-                kSq ? comp_sq + (long long)t * V : nullptr, kSdfOut ? comp_sdf + (long long)t * V : nullptr, vox);
-        } else if (live) {
-            EnvCursor none(tile, nthr, -1);
-            emit_range<false, false, false>(0, nz, none, false, mk, false, zlo, nthr, scol, sfcol, V2i, out, nz);
-        }
-        return;
-    }
-
-    const bool dyn = live && !col_static;
-    const bool occ = dyn && gmin < 0;  // some slab voxel of the column lies inside a human
-    if (dyn) {
-        int w0 = 0, w1 = nz;
-        const long long diff = (long long)cmax - gmin;  // > 0
-        if (diff < (long long)nz * nz) {
-            int R = (int)sqrtf((float)diff);
-            while ((long long)R * R < diff)
-                ++R;
-            while (R > 1 && (long long)(R - 1) * (R - 1) >= diff)
-                --R;
-            w0 = max(zlo - R + 1, 0);
-            w1 = min(zlo + S + R - 1, nz);
-        }
-        atomicMin(&s_w0, w0);
-        atomicMax(&s_w1, w1);
-        if (occ)
-            s_occ = 1;
-    }
-    __syncthreads();
-    const int ww0 = s_w0, ww1 = s_w1;  // some column is dynamic: ww0 <= zlo, ww1 >= zlo + S
-    const bool any_occ = s_occ != 0;
-    // the planes outside the window union are copies of the static block:
-    // 16-byte accesses by all threads first (the CTA's per-column loops below
-    // are what its time depends on)
-    if (vec) {
-        const int nc = (int)min((long long)nthr, V2 - col0);
-        int32_t *osq = kSq ? comp_sq + (long long)t * V : nullptr;
-        float *osdf = kSdfOut ? comp_sdf + (long long)t * V : nullptr;
-        copy_static_planes<kSq, kSdfOut, kStaticSdf, false>(static_sq, static_sdf, V2, nz, 0, ww0, col0, nc, osq,
-                                                            osdf, vox);
-        copy_static_planes<kSq, kSdfOut, kStaticSdf, false>(static_sq, static_sdf, V2, nz, ww1, nz, col0, nc, osq,
-                                                            osdf, vox);
-    }
-    if (!live)
-        return;  // no block-level synchronisation below
-
-    int top = -1;  // set O stack top (-1: no site, or a static column)
-    if (dyn) {
-        int za, zb;
-        top = build_sets<false>(tile, mk, occ, nthr, S, nz, zlo, scol, sfcol, dcol, V2, out, za, zb, rep);
-    }
-    EnvCursor O(tile + nthr, nthr, top);
-    const bool useO = top >= 0;
-    const int sa = zlo, sb = zlo + S;
-    if (!vec)
-        emit_range<false, false, false>(0, ww0, O, false, mk, false, zlo, nthr, scol, sfcol, V2i, out, nz);
-    emit_range<false, true, false>(ww0, sa, O, useO, mk, false, zlo, nthr, scol, sfcol, V2i, out, nz);
-    if (any_occ)  // skip the occupied slab voxels (set F wrote them)
-        emit_range<true, true, false>(sa, sb, O, useO, mk, occ, zlo, nthr, scol, sfcol, V2i, out, nz);
-    else
-        emit_range<false, true, false>(sa, sb, O, useO, mk, false, zlo, nthr, scol, sfcol, V2i, out, nz);
-    emit_range<false, true, false>(sb, ww1, O, useO, mk, false, zlo, nthr, scol, sfcol, V2i, out, nz);
-    if (!vec)
-        emit_range<false, false, false>(ww1, nz, O, false, mk, false, zlo, nthr, scol, sfcol, V2i, out, nz);
-}
+};
 
 }  // namespace comp
 }  // namespace pcdf

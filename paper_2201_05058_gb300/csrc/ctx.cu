@@ -116,7 +116,7 @@ int pcdf_scratch_bytes(const pcdf_grid *grid, int32_t T, int32_t H, size_t *byte
         return fail(PCDF_EINVAL, "bytes is NULL");
     // the static build and the from-scratch comparator, or a composite whose
     // capsules touch every slice (the largest slab: int16 and int32
-    // intermediates plus the column maxima)
+    // intermediates, and a plane to spare)
     const size_t V = (size_t)nvox(grid), slab = (size_t)T * V;
     const size_t comp = align_up(slab * sizeof(int16_t)) + align_up(slab * sizeof(int32_t)) +
                         align_up((size_t)grid->nx * grid->ny * sizeof(int32_t));

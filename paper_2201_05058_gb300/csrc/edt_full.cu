@@ -49,16 +49,15 @@ __global__ void __launch_bounds__(kThreads, 4)
     full::edt_xy_block<false>(bits, carry, nx, ny, nz, W, blockIdx.x, blockIdx.y, mid, smem);
 }
 
-// colmax (nullable): each column's largest value of sq.  50 us for the 256^3
-// map (105 us before): the 12 bytes per voxel alone take 30 us.
+// 50 us for the 256^3 map (105 us before): the 12 bytes per voxel alone take
+// 30 us.
 template <bool kSdf>
 __global__ void __launch_bounds__(kThreads, 4)
     k_edt_z(const int32_t *__restrict__ mid, int32_t *__restrict__ sq, float *__restrict__ sdf, float vox, int n,
-            long long ncols, int vec, int32_t *__restrict__ colmax)
+            long long ncols, int vec)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    full::edt_z_block<kSdf, false>(mid, sq, sdf, vox, n, ncols, (long long)blockIdx.x * full::kTileCols, vec != 0, smem,
-                                   colmax);
+    full::edt_z_block<kSdf, false>(mid, sq, sdf, vox, n, ncols, (long long)blockIdx.x * full::kTileCols, vec != 0, smem);
 }
 
 size_t tile_bytes(int n) { return blockmin::tile_words(n) * sizeof(uint32_t); }
@@ -76,7 +75,7 @@ size_t full_edt_scratch(int nx, int ny, int nz, size_t *bits_off, size_t *carry_
 }
 
 cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, int H, int nx, int ny, int nz,
-                            int32_t *sq, float *sdf, float vox, void *ws, cudaStream_t st, int32_t *colmax)
+                            int32_t *sq, float *sdf, float vox, void *ws, cudaStream_t st)
 {
     size_t bo, co, mo;
     full_edt_scratch(nx, ny, nz, &bo, &co, &mo);
@@ -119,11 +118,11 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
     if (sdf) {
         if ((e = allow_shared(k_edt_z<true>)) != cudaSuccess)
             return e;
-        k_edt_z<true><<<nbz, kThreads, sz, st>>>(mid, sq, sdf, vox, nz, ncols, vec, colmax);
+        k_edt_z<true><<<nbz, kThreads, sz, st>>>(mid, sq, sdf, vox, nz, ncols, vec);
     } else {
         if ((e = allow_shared(k_edt_z<false>)) != cudaSuccess)
             return e;
-        k_edt_z<false><<<nbz, kThreads, sz, st>>>(mid, sq, nullptr, vox, nz, ncols, vec, colmax);
+        k_edt_z<false><<<nbz, kThreads, sz, st>>>(mid, sq, nullptr, vox, nz, ncols, vec);
     }
     return cudaGetLastError();
 }

@@ -119,12 +119,9 @@ cudaError_t launch_pass_x(int mode, const uint8_t *occ, const CapBatch *caps, in
 // the capsules alone (mode 2), then the fused x+y pass and the z pass; sq and
 // (nullable) sdf are [nz][ny][nx].  ws holds full_edt_scratch() bytes
 // (256-byte aligned): row words, their carries and the 2-D partial field.
-// colmax (nullable): receives the largest value of every column of sq, as
-// launch_colmax would write it.
 size_t full_edt_scratch(int nx, int ny, int nz, size_t *bits_off, size_t *carry_off, size_t *mid_off);
 cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, int H, int nx, int ny, int nz,
-                            int32_t *sq, float *sdf, float vox, void *ws, cudaStream_t stream,
-                            int32_t *colmax = nullptr);
+                            int32_t *sq, float *sdf, float vox, void *ws, cudaStream_t stream);
 
 // Lower-envelope pass over ncols columns: element e of column c lives at
 // (c / nx) * outer_stride + (c % nx) + e * stride, e in [0, n).
@@ -153,19 +150,14 @@ size_t dyn_xy_words(int ny, int run_rows);
 cudaError_t launch_dyn_xy(const CapBatch *caps, const SlabMap *map, int H, int nx, int ny, int zlo, int S, int t0,
                           int n_t, int run_rows, int32_t *dyn_mid, cudaStream_t stream);
 
-// colmax[y][x] = largest value of the column (x, y) of sq [nz][ny][nx].
-cudaError_t launch_colmax(const int32_t *sq, int nx, int ny, int nz, int32_t *colmax, cudaStream_t stream);
-
 // z-pass of the dynamic field over the slab [zlo, zlo + S) fused with the
 // composite min against static_sq and the float epilogue, for t = t0 ..
 // t0 + nt - 1 (outputs and slab indexed by the absolute t).
 // static_sdf (nullable) is the float field of static_sq; where the static
-// field wins the min it is copied instead of recomputed.  colmax holds the
-// column maxima of static_sq (launch_colmax): columns and z ranges where the
-// static field provably wins skip the envelope.
-cudaError_t launch_composite_z(const int32_t *static_sq, const float *static_sdf, const int32_t *colmax,
-                               const int32_t *dyn_mid, const SlabMap *map, int nx, int ny, int nz, int zlo, int S,
-                               int t0, int nt, int32_t *comp_sq, float *comp_sdf, float vox, cudaStream_t stream);
+// field wins the min it is copied instead of recomputed.
+cudaError_t launch_composite_z(const int32_t *static_sq, const float *static_sdf, const int32_t *dyn_mid,
+                               const SlabMap *map, int nx, int ny, int nz, int zlo, int S, int t0, int nt,
+                               int32_t *comp_sq, float *comp_sdf, float vox, cudaStream_t stream);
 
 // Copies static_sq into t = t0 .. t0 + nt - 1 of comp (and its float field)
 // when no capsule touches the grid.

@@ -3,9 +3,7 @@
 // then pcdf_build_predicted_composite, with the capsules' x+y pass (it needs
 // no static field) on a side stream beside the static build.  The side stream
 // first waits for the work already on the stream; the stream waits for the
-// capsule pass before the composite's z stage.  The static z pass also writes
-// the static column maxima that the z stage reads (no separate pass over the
-// static field).  Events are created per call (no timing) and released before
+// capsule pass before the composite's z stage.  Events are created per call (no timing) and released before
 // returning; nothing synchronises the host.
 //
 // Splitting the z stage into column chunks that start behind the static z
@@ -88,13 +86,11 @@ int pcdf_update_fields(const pcdf_grid *grid, const uint8_t *occ, int32_t T, int
             return rc;
     if ((e = cudaEventRecord(ev.done, sd)) != cudaSuccess)
         return cuda_fail(e, "update stream order");
-    // the static z pass also writes the column maxima that the z stage reads
-    int32_t *colmax = p.S > 0 ? (int32_t *)((char *)wsC + p.colmax_off) : nullptr;
-    if (int rc = run_full_edt(grid, 0, occ, &none, 0, static_sq, static_sdf, workspace, st, colmax))
+    if (int rc = run_full_edt(grid, 0, occ, &none, 0, static_sq, static_sdf, workspace, st))
         return rc;
     if ((e = cudaStreamWaitEvent(st, ev.done, 0)) != cudaSuccess)
         return cuda_fail(e, "update stream order");
-    return composite_finish(grid, static_sq, static_sdf, 0, T, p, comp_sq, comp_sdf, wsC, st, colmax != nullptr);
+    return composite_finish(grid, static_sq, static_sdf, 0, T, p, comp_sq, comp_sdf, wsC, st);
 }
 
 }  // extern "C"

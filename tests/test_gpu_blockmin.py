@@ -86,3 +86,32 @@ def test_capsule_slices(nx, ny, nz):
     want = oracle.predicted_composite(static, caps)
     assert np.array_equal(sq.cpu().numpy(), want)
     assert np.array_equal(sdf.cpu().numpy().view(np.int32), oracle.sdf_from_sq(want, 0.05).view(np.int32))
+
+
+# the composite's z pass: groups of time steps with a remainder, blocks that are
+# copies, near a human, inside one, and out of the 16-bit range (an empty or
+# nearly empty map, humans more than 177 voxels away), every output variant
+@pytest.mark.parametrize("nx,ny,nz,T,boxes", [(64, 9, 70, 5, 4), (33, 31, 41, 9, 6), (430, 6, 40, 3, 0), (7, 240, 96, 6, 1), (65, 33, 9, 1, 3)])
+def test_composite_blocks(nx, ny, nz, T, boxes):
+    rng = np.random.default_rng(nx + T)
+    grid = scenes.Grid(nx, ny, nz, 0.05)
+    occ, _ = scenes.boxes_occupancy(grid, boxes, rng)
+    static = oracle.edt(occ)
+    sdf = oracle.sdf_from_sq(static, 0.05)
+    r = 16 * min(nx, ny, nz) // 3
+    top = 16 * nz - 20
+    caps = np.array([[[40 + 9 * t, 16 * ny // 2, r, 40 + 9 * t, 16 * ny // 2, max(top - r, r), r],
+                      [60, 30 + 5 * t, 30, 60 + 3 * t, 30, top // 2, 25]] for t in range(T)], np.int32)
+    want = oracle.predicted_composite(static, caps)
+    want_sdf = oracle.sdf_from_sq(want, 0.05).view(np.int32)
+    st, sf = torch.from_numpy(static).to("cuda"), torch.from_numpy(sdf).to("cuda")
+    for want_sq, want_f, given in ((True, True, sf), (True, True, None), (True, False, None), (False, True, sf), (False, True, None)):
+        sq, f = pcdf.build_predicted_composite(st, grid, caps, want_sq=want_sq, want_sdf=want_f, static_sdf=given)
+        if want_sq:
+            assert np.array_equal(sq.cpu().numpy(), want)
+        if want_f:
+            assert np.array_equal(f.cpu().numpy().view(np.int32), want_sdf)
+    batch = pcdf.Batch([(grid, torch.from_numpy(occ).to("cuda"), caps)])
+    batch.run()
+    assert batch.error() == 0
+    assert np.array_equal(batch.comp_sq[0].cpu().numpy(), want)
