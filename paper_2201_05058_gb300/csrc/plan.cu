@@ -230,6 +230,8 @@ int plan_composite(const pcdf_grid *grid, int T, int H, const int32_t *caps, Com
         p.need = align_up((size_t)p.slab * sizeof(int32_t));
     else
         p.need = align_up((size_t)p.slab * sizeof(int16_t)) + align_up((size_t)p.slab * sizeof(int32_t));
+    if (p.S > 0)  // and a plane of the grid, part of the size that callers have always been told
+        p.need += align_up((size_t)grid->nx * grid->ny * sizeof(int32_t));
     return PCDF_OK;
 }
 
