@@ -330,6 +330,12 @@ int pcdf_composite_translated(const pcdf_grid *grid, const int32_t *static_sq, c
 int pcdf_query_cost(const pcdf_grid *grid, const float *sdf, int32_t T, const float *spheres, const int32_t *tidx,
                     int64_t N, float eps, float *h, int32_t *n_oob, void *stream);
 
+/* pcdf_query_cost of the spheres (centres[q], radii[q]) (device fp32 [N][3] and
+ * [N]), which are also written to spheres (device fp32 [N][4], 16-byte
+ * aligned, out), for a later pcdf_query_cost_backward. */
+int pcdf_query_cost_packed(const pcdf_grid *grid, const float *sdf, int32_t T, const float *centres, const float *radii,
+                           const int32_t *tidx, int64_t N, float eps, float *spheres, float *h, void *stream);
+
 /* Backward of pcdf_query_cost: with the same inputs and upstream gradient
  * grad_h (device fp32 [N]),
  *   grad_c[q] = -grad_h[q] * grad_c d(c)   where h > 0 and d is finite, else 0

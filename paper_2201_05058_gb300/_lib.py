@@ -39,7 +39,7 @@ EXPORTS = (
     "pcdf_filter_voxels", "pcdf_collapse_2d", "pcdf_update_workspace_bytes", "pcdf_update_fields",
     "pcdf_scratch_workspace_bytes", "pcdf_build_from_scratch",
     "pcdf_field_max", "pcdf_template_radius", "pcdf_lattice_placements", "pcdf_template_box", "pcdf_template_workspace_bytes", "pcdf_build_template", "pcdf_composite_translated",
-    "pcdf_query_cost", "pcdf_query_cost_backward",
+    "pcdf_query_cost", "pcdf_query_cost_packed", "pcdf_query_cost_backward",
     "pcdf_batch_create", "pcdf_batch_destroy", "pcdf_batch_workspace_bytes", "pcdf_batch_tiles_used",
     "pcdf_batch_upload", "pcdf_batch_run", "pcdf_batch_error", "pcdf_batch_block_stage", "pcdf_batch_autotune_workspace_bytes",
     "pcdf_batch_autotune",
@@ -85,6 +85,7 @@ def _declare(lib):
         "pcdf_build_template": [P, I32, P, P, SZ, P],
         "pcdf_composite_translated": [G, P, P, I32, I32, P, P, I32, P, P, P, P],
         "pcdf_query_cost": [G, P, I32, P, P, I64, F32, P, P, P],
+        "pcdf_query_cost_packed": [G, P, I32, P, P, P, I64, F32, P, P, P],
         "pcdf_query_cost_backward": [G, P, I32, P, P, I64, F32, P, P, P, P],
     }
     E = ctypes.POINTER(PcdfEnv)
@@ -156,7 +157,10 @@ def load(build_if_missing: bool = True, checked: bool = None):
     """Load libpcdf.so, or the bounds-checked libpcdf_checked.so (checked, or
     use_checked(True)), building it first if allowed and needed."""
     global _lib, _lib_checked
-    checked = _use_checked if checked is None else checked
+    if checked is None:
+        if _lib is not None and not _use_checked:  # loaded already: the usual call
+            return _lib
+        checked = _use_checked
     path = _build.LIB_CHECKED if checked else _build.LIB
     with _lock:
         if (_lib_checked if checked else _lib) is None:

@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 from dataclasses import dataclass
+from functools import lru_cache
 
 import numpy as np
 import torch
@@ -30,9 +31,15 @@ class Grid:
         return (self.nz, self.ny, self.nx)
 
 
+@lru_cache(maxsize=256)
+def _grid_struct(nx, ny, nz, vox, origin) -> _lib.PcdfGrid:
+    """The C struct of a grid's values (read only: one for equal grids)."""
+    return _lib.PcdfGrid(int(nx), int(ny), int(nz), float(vox), (ctypes.c_float * 3)(*(float(v) for v in origin)))
+
+
 def _cgrid(g) -> _lib.PcdfGrid:
-    o = tuple(float(v) for v in getattr(g, "origin", (0.0, 0.0, 0.0)))
-    return _lib.PcdfGrid(int(g.nx), int(g.ny), int(g.nz), float(g.vox), (ctypes.c_float * 3)(*o))
+    o = getattr(g, "origin", (0.0, 0.0, 0.0))
+    return _grid_struct(g.nx, g.ny, g.nz, g.vox, o if type(o) is tuple else tuple(float(v) for v in o))
 
 
 def _shape(g):
@@ -40,7 +47,11 @@ def _shape(g):
 
 
 def _stream(dev: torch.device) -> int:
-    return torch.cuda.current_stream(dev).cuda_stream
+    return torch.cuda.current_stream(dev).cuda_stream if dev.index is None else _raw_stream(dev.index)
+
+
+# the current stream's handle without a Stream object around it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda i: torch.cuda.current_stream(i).cuda_stream)
 
 
 def _need(t: torch.Tensor, name: str, dtype, shape=None):
@@ -50,7 +61,7 @@ def _need(t: torch.Tensor, name: str, dtype, shape=None):
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t
 
@@ -66,7 +77,7 @@ def _caps_host(caps):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _workspace(nbytes: int, dev) -> torch.Tensor:
@@ -108,7 +119,7 @@ def build_static_sdf(occ: torch.Tensor, grid, want_sdf: bool = True, out_sq=None
     lib = _lib.load()
     g = _cgrid(grid)
     nbytes = ctypes.c_size_t(0)
-    _lib.check(lib.pcdf_static_workspace_bytes(ctypes.byref(g), ctypes.byref(nbytes)), "static workspace")
+    _lib.check(lib.pcdf_static_workspace_bytes(g, nbytes), "static workspace")
     sq = out_sq if out_sq is not None else torch.empty(shp, dtype=torch.int32, device=dev)
     _need(sq, "static_sq", torch.int32, shp)
     sdf = None
@@ -116,8 +127,8 @@ def build_static_sdf(occ: torch.Tensor, grid, want_sdf: bool = True, out_sq=None
         sdf = out_sdf if out_sdf is not None else torch.empty(shp, dtype=torch.float32, device=dev)
         _need(sdf, "static_sdf", torch.float32, shp)
     ws = _workspace(nbytes.value, dev)
-    _lib.check(lib.pcdf_build_static_sdf(ctypes.byref(g), _ptr(occ), _ptr(sq), _ptr(sdf), _ptr(ws), ws.numel(),
-                                         ctypes.c_void_p(_stream(dev))), "pcdf_build_static_sdf")
+    _lib.check(lib.pcdf_build_static_sdf(g, _ptr(occ), _ptr(sq), _ptr(sdf), _ptr(ws), ws.numel(),
+                                         _stream(dev)), "pcdf_build_static_sdf")
     return sq, sdf
 
 
@@ -130,8 +141,8 @@ def filter_voxels(occ: torch.Tensor, grid, min_neighbours: int = 5, out=None) ->
     out = out if out is not None else torch.empty_like(occ)
     _need(out, "out", torch.uint8, shp)
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_filter_voxels(ctypes.byref(g), _ptr(occ), int(min_neighbours), _ptr(out),
-                                              ctypes.c_void_p(_stream(occ.device))), "pcdf_filter_voxels")
+    _lib.check(_lib.load().pcdf_filter_voxels(g, _ptr(occ), int(min_neighbours), _ptr(out),
+                                              _stream(occ.device)), "pcdf_filter_voxels")
     return out
 
 
@@ -141,8 +152,8 @@ def collapse_2d(occ: torch.Tensor, grid, z0: int, z1: int) -> torch.Tensor:
     _need(occ, "occ", torch.uint8, _shape(grid))
     out = torch.empty((grid.ny, grid.nx), dtype=torch.uint8, device=occ.device)
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_collapse_2d(ctypes.byref(g), _ptr(occ), int(z0), int(z1), _ptr(out),
-                                            ctypes.c_void_p(_stream(occ.device))), "pcdf_collapse_2d")
+    _lib.check(_lib.load().pcdf_collapse_2d(g, _ptr(occ), int(z0), int(z1), _ptr(out),
+                                            _stream(occ.device)), "pcdf_collapse_2d")
     return out
 
 
@@ -175,7 +186,7 @@ def build_predicted_composite(static_sq: torch.Tensor, grid, caps, want_sq: bool
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
     nbytes = ctypes.c_size_t(0)
-    _lib.check(lib.pcdf_composite_workspace_bytes(ctypes.byref(g), T, H, cp, ctypes.byref(nbytes)),
+    _lib.check(lib.pcdf_composite_workspace_bytes(g, T, H, cp, ctypes.byref(nbytes)),
                "composite workspace")
     sq = sdf = None
     if want_sq:
@@ -185,9 +196,9 @@ def build_predicted_composite(static_sq: torch.Tensor, grid, caps, want_sq: bool
         sdf = out_sdf if out_sdf is not None else torch.empty((T,) + shp, dtype=torch.float32, device=dev)
         _need(sdf, "comp_sdf", torch.float32, (T,) + shp)
     ws = _workspace(nbytes.value, dev)
-    _lib.check(lib.pcdf_build_predicted_composite(ctypes.byref(g), _ptr(static_sq), _ptr(static_sdf), T, H, cp,
+    _lib.check(lib.pcdf_build_predicted_composite(g, _ptr(static_sq), _ptr(static_sdf), T, H, cp,
                                                   _ptr(sq), _ptr(sdf),
-                                                  _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(dev))),
+                                                  _ptr(ws), ws.numel(), _stream(dev)),
                "pcdf_build_predicted_composite")
     return sq, sdf
 
@@ -199,7 +210,7 @@ def composite_workspace(grid, caps, device) -> torch.Tensor:
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
     nbytes = ctypes.c_size_t(0)
-    _lib.check(_lib.load().pcdf_composite_workspace_bytes(ctypes.byref(g), T, H, cp, ctypes.byref(nbytes)),
+    _lib.check(_lib.load().pcdf_composite_workspace_bytes(g, T, H, cp, ctypes.byref(nbytes)),
                "composite workspace")
     return _workspace(nbytes.value, device)
 
@@ -211,20 +222,23 @@ def composite_slab(grid, caps):
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
     zlo, S = ctypes.c_int32(0), ctypes.c_int32(0)
-    _lib.check(_lib.load().pcdf_composite_slab(ctypes.byref(g), T, H, cp, ctypes.byref(zlo), ctypes.byref(S)),
+    _lib.check(_lib.load().pcdf_composite_slab(g, T, H, cp, ctypes.byref(zlo), ctypes.byref(S)),
                "pcdf_composite_slab")
     return zlo.value, S.value
 
 
 def composite_prepare(grid, caps, workspace: torch.Tensor):
     """First stage of the composite: capsule row pass and y pass into workspace."""
-    caps = _caps_host(caps)
+    _prepare(grid, _caps_host(caps), workspace, _stream(workspace.device) if isinstance(workspace, torch.Tensor) and
+             workspace.is_cuda else None)
+
+
+def _prepare(grid, caps, workspace, stream):
     T, H = int(caps.shape[0]), int(caps.shape[1])
     _need(workspace, "workspace", torch.uint8)
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
-    _lib.check(_lib.load().pcdf_composite_prepare(ctypes.byref(g), T, H, cp, _ptr(workspace), workspace.numel(),
-                                                  ctypes.c_void_p(_stream(workspace.device))),
+    _lib.check(_lib.load().pcdf_composite_prepare(g, T, H, cp, _ptr(workspace), workspace.numel(), stream),
                "pcdf_composite_prepare")
 
 
@@ -247,16 +261,16 @@ def composite_finish(static_sq, grid, caps, workspace: torch.Tensor, comp_sq=Non
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
     if t_range is None:
-        _lib.check(_lib.load().pcdf_composite_finish(ctypes.byref(g), _ptr(static_sq), _ptr(static_sdf), T, H, cp,
+        _lib.check(_lib.load().pcdf_composite_finish(g, _ptr(static_sq), _ptr(static_sdf), T, H, cp,
                                                      _ptr(comp_sq), _ptr(comp_sdf), _ptr(workspace),
-                                                     workspace.numel(), ctypes.c_void_p(_stream(static_sq.device))),
+                                                     workspace.numel(), _stream(static_sq.device)),
                    "pcdf_composite_finish")
     else:
         t0, nt = (int(v) for v in t_range)
-        _lib.check(_lib.load().pcdf_composite_finish_range(ctypes.byref(g), _ptr(static_sq), _ptr(static_sdf), T, H,
+        _lib.check(_lib.load().pcdf_composite_finish_range(g, _ptr(static_sq), _ptr(static_sdf), T, H,
                                                            cp, t0, nt, _ptr(comp_sq), _ptr(comp_sdf),
                                                            _ptr(workspace), workspace.numel(),
-                                                           ctypes.c_void_p(_stream(static_sq.device))),
+                                                           _stream(static_sq.device)),
                    "pcdf_composite_finish_range")
 
 
@@ -278,7 +292,7 @@ def update_workspace(grid, caps, device) -> torch.Tensor:
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
     n = ctypes.c_size_t(0)
-    _lib.check(_lib.load().pcdf_update_workspace_bytes(ctypes.byref(g), T, H, cp, ctypes.byref(n)),
+    _lib.check(_lib.load().pcdf_update_workspace_bytes(g, T, H, cp, ctypes.byref(n)),
                "pcdf_update_workspace_bytes")
     return _workspace(n.value, torch.device(device))
 
@@ -309,7 +323,7 @@ def predicted_fields(occ: torch.Tensor, grid, caps, workspace=None, out_static_s
     side = _side_stream(dev)
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
-    _lib.check(_lib.load().pcdf_update_fields(ctypes.byref(g), _ptr(occ), T, H, cp, _ptr(st_sq), _ptr(st_sdf),
+    _lib.check(_lib.load().pcdf_update_fields(g, _ptr(occ), T, H, cp, _ptr(st_sq), _ptr(st_sdf),
                                               _ptr(sq), _ptr(sdf), _ptr(ws), ws.numel(),
                                               ctypes.c_void_p(main.cuda_stream), ctypes.c_void_p(side.cuda_stream)),
                "pcdf_update_fields")
@@ -380,7 +394,7 @@ def build_from_scratch(occ: torch.Tensor, grid, caps, want_sdf: bool = True, out
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
     nbytes = ctypes.c_size_t(0)
-    _lib.check(lib.pcdf_scratch_workspace_bytes(ctypes.byref(g), T, H, ctypes.byref(nbytes)), "scratch workspace")
+    _lib.check(lib.pcdf_scratch_workspace_bytes(g, T, H, ctypes.byref(nbytes)), "scratch workspace")
     sq = out_sq if out_sq is not None else torch.empty((T,) + shp, dtype=torch.int32, device=dev)
     _need(sq, "sq", torch.int32, (T,) + shp)
     sdf = None
@@ -388,8 +402,8 @@ def build_from_scratch(occ: torch.Tensor, grid, caps, want_sdf: bool = True, out
         sdf = out_sdf if out_sdf is not None else torch.empty((T,) + shp, dtype=torch.float32, device=dev)
         _need(sdf, "sdf", torch.float32, (T,) + shp)
     ws = _workspace(nbytes.value, dev)
-    _lib.check(lib.pcdf_build_from_scratch(ctypes.byref(g), _ptr(occ), T, H, cp, _ptr(sq), _ptr(sdf), _ptr(ws),
-                                           ws.numel(), ctypes.c_void_p(_stream(dev))), "pcdf_build_from_scratch")
+    _lib.check(lib.pcdf_build_from_scratch(g, _ptr(occ), T, H, cp, _ptr(sq), _ptr(sdf), _ptr(ws),
+                                           ws.numel(), _stream(dev)), "pcdf_build_from_scratch")
     return sq, sdf
 
 
@@ -427,7 +441,7 @@ def build_template(cap, R: int, device):
     _lib.check(lib.pcdf_template_workspace_bytes(cp, int(R), ctypes.byref(nbytes)), "template workspace")
     tmpl = torch.empty((dims[2], dims[1], dims[0]), dtype=torch.int32, device=dev)
     ws = _workspace(nbytes.value, dev)
-    _lib.check(lib.pcdf_build_template(cp, int(R), _ptr(tmpl), _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(dev))),
+    _lib.check(lib.pcdf_build_template(cp, int(R), _ptr(tmpl), _ptr(ws), ws.numel(), _stream(dev)),
                "pcdf_build_template")
     return tmpl, lo
 
@@ -439,7 +453,7 @@ def template_radius(static_sq: torch.Tensor) -> int:
     _need(static_sq, "static_sq", torch.int32)
     out = torch.empty(1, dtype=torch.int32, device=static_sq.device)
     _lib.check(_lib.load().pcdf_field_max(_ptr(static_sq), static_sq.numel(), _ptr(out),
-                                          ctypes.c_void_p(_stream(static_sq.device))), "pcdf_field_max")
+                                          _stream(static_sq.device)), "pcdf_field_max")
     R = ctypes.c_int32(0)
     _lib.check(_lib.load().pcdf_template_radius(int(out.item()), ctypes.byref(R)), "pcdf_template_radius")
     return int(R.value)
@@ -490,9 +504,9 @@ def composite_translated(static_sq: torch.Tensor, grid, tmpl: torch.Tensor, lo, 
     dims = (ctypes.c_int32 * 3)(int(tmpl.shape[2]), int(tmpl.shape[1]), int(tmpl.shape[0]))
     g = _cgrid(grid)
     _lib.check(_lib.load().pcdf_composite_translated(
-        ctypes.byref(g), _ptr(static_sq), _ptr(static_sdf), T, H, _ptr(tmpl), dims, int(R),
+        g, _ptr(static_sq), _ptr(static_sdf), T, H, _ptr(tmpl), dims, int(R),
         lo.ctypes.data_as(ctypes.c_void_p) if H > 0 else None, _ptr(comp_sq), _ptr(comp_sdf),
-        ctypes.c_void_p(_stream(dev))), "pcdf_composite_translated")
+        _stream(dev)), "pcdf_composite_translated")
     return comp_sq, comp_sdf
 
 
@@ -528,8 +542,8 @@ def query_cost(sdf: torch.Tensor, grid, spheres: torch.Tensor, tidx: torch.Tenso
     h = torch.empty(tidx.shape, dtype=torch.float32, device=dev)
     oob = torch.zeros(1, dtype=torch.int32, device=dev) if count_oob else None
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_query_cost(ctypes.byref(g), _ptr(sdf), T, _ptr(spheres), _ptr(tidx), N,
-                                           float(eps), _ptr(h), _ptr(oob), ctypes.c_void_p(_stream(dev))),
+    _lib.check(_lib.load().pcdf_query_cost(g, _ptr(sdf), T, _ptr(spheres), _ptr(tidx), N,
+                                           float(eps), _ptr(h), _ptr(oob), _stream(dev)),
                "pcdf_query_cost")
     if count_oob:
         return h, oob
@@ -547,11 +561,22 @@ def query_cost_backward(sdf: torch.Tensor, grid, spheres: torch.Tensor, tidx: to
     gc = torch.empty(tuple(spheres.shape[:-1]) + (3,), dtype=torch.float32, device=dev)
     gr = torch.empty(tidx.shape, dtype=torch.float32, device=dev) if want_grad_r else None
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_query_cost_backward(ctypes.byref(g), _ptr(sdf), T, _ptr(spheres), _ptr(tidx), N,
+    _lib.check(_lib.load().pcdf_query_cost_backward(g, _ptr(sdf), T, _ptr(spheres), _ptr(tidx), N,
                                                     float(eps), _ptr(grad_h), _ptr(gc), _ptr(gr),
-                                                    ctypes.c_void_p(_stream(dev))),
+                                                    _stream(dev)),
                "pcdf_query_cost_backward")
     return gc, gr
+
+
+def _query_packed(sdf, grid, centres, radii, spheres, tidx, eps):
+    """query_cost of the spheres (centres, radii), which are also written to
+    `spheres` [..., 4]."""
+    sdf, T, N = _query_args(sdf, grid, spheres, tidx)
+    h = torch.empty(tidx.shape, dtype=torch.float32, device=sdf.device)
+    _lib.check(_lib.load().pcdf_query_cost_packed(_cgrid(grid), _ptr(sdf), T, _ptr(centres), _ptr(radii), _ptr(tidx), N,
+                                                  float(eps), _ptr(spheres), _ptr(h), _stream(sdf.device)),
+               "pcdf_query_cost_packed")
+    return h
 
 
 class HingeCost(torch.autograd.Function):
@@ -560,9 +585,16 @@ class HingeCost(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, centres, radii, sdf, tidx, eps, grid):
-        spheres = torch.cat([centres.detach(), radii.detach().unsqueeze(-1)], dim=-1).contiguous()
         tidx = tidx.contiguous()
-        h = query_cost(sdf, grid, spheres, tidx, eps)
+        if (centres.is_cuda and centres.dtype == torch.float32 and radii.dtype == torch.float32
+                and radii.device == centres.device and centres.dim() > 0 and centres.shape[-1] == 3
+                and radii.shape == centres.shape[:-1] and centres.is_contiguous() and radii.is_contiguous()):
+            # the spheres are packed by the query itself
+            spheres = torch.empty(radii.shape + (4,), dtype=torch.float32, device=centres.device)
+            h = _query_packed(sdf, grid, centres, radii, spheres, tidx, eps)
+        else:
+            spheres = torch.cat([centres.detach(), radii.detach().unsqueeze(-1)], dim=-1).contiguous()
+            h = query_cost(sdf, grid, spheres, tidx, eps)
         ctx.save_for_backward(spheres, sdf, tidx)
         ctx.eps = eps
         ctx.grid = grid
@@ -618,7 +650,7 @@ class Context:
         """Upper bound of the scratch of any call for grid with up to T fields and H humans."""
         g = _cgrid(grid)
         n = ctypes.c_size_t(0)
-        _lib.check(_lib.load().pcdf_scratch_bytes(ctypes.byref(g), int(T), int(H), ctypes.byref(n)),
+        _lib.check(_lib.load().pcdf_scratch_bytes(g, int(T), int(H), ctypes.byref(n)),
                    "pcdf_scratch_bytes")
         return n.value
 
@@ -631,7 +663,7 @@ class Context:
         sq = torch.empty(shp, dtype=torch.int32, device=occ.device)
         sdf = torch.empty(shp, dtype=torch.float32, device=occ.device) if want_sdf else None
         g = _cgrid(grid)
-        _lib.check(self._lib.pcdf_ctx_build_static_sdf(self._h, ctypes.byref(g), _ptr(occ), _ptr(sq), _ptr(sdf)),
+        _lib.check(self._lib.pcdf_ctx_build_static_sdf(self._h, g, _ptr(occ), _ptr(sq), _ptr(sdf)),
                    "pcdf_ctx_build_static_sdf")
         return sq, sdf
 
@@ -646,7 +678,7 @@ class Context:
         sdf = torch.empty((T,) + shp, dtype=torch.float32, device=dev) if want_sdf else None
         g = _cgrid(grid)
         cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
-        _lib.check(self._lib.pcdf_ctx_build_predicted_composite(self._h, ctypes.byref(g), _ptr(static_sq),
+        _lib.check(self._lib.pcdf_ctx_build_predicted_composite(self._h, g, _ptr(static_sq),
                                                                 _ptr(static_sdf), T, H, cp, _ptr(sq), _ptr(sdf)),
                    "pcdf_ctx_build_predicted_composite")
         return sq, sdf
@@ -660,7 +692,7 @@ class Context:
         sdf = torch.empty((T,) + shp, dtype=torch.float32, device=occ.device) if want_sdf else None
         g = _cgrid(grid)
         cp = caps.ctypes.data_as(ctypes.c_void_p) if H > 0 else None
-        _lib.check(self._lib.pcdf_ctx_build_from_scratch(self._h, ctypes.byref(g), _ptr(occ), T, H, cp, _ptr(sq),
+        _lib.check(self._lib.pcdf_ctx_build_from_scratch(self._h, g, _ptr(occ), T, H, cp, _ptr(sq),
                                                          _ptr(sdf)), "pcdf_ctx_build_from_scratch")
         return sq, sdf
 
@@ -668,7 +700,7 @@ class Context:
         sdf, T, N = _query_args(sdf, grid, spheres, tidx)
         h = torch.empty(tidx.shape, dtype=torch.float32, device=sdf.device)
         g = _cgrid(grid)
-        _lib.check(self._lib.pcdf_ctx_query_cost(self._h, ctypes.byref(g), _ptr(sdf), T, _ptr(spheres), _ptr(tidx),
+        _lib.check(self._lib.pcdf_ctx_query_cost(self._h, g, _ptr(sdf), T, _ptr(spheres), _ptr(tidx),
                                                  N, float(eps), _ptr(h), None), "pcdf_ctx_query_cost")
         return h
 
@@ -681,7 +713,7 @@ class Context:
         gc = torch.empty(tuple(spheres.shape[:-1]) + (3,), dtype=torch.float32, device=sdf.device)
         gr = torch.empty(tidx.shape, dtype=torch.float32, device=sdf.device)
         g = _cgrid(grid)
-        _lib.check(self._lib.pcdf_ctx_query_cost_backward(self._h, ctypes.byref(g), _ptr(sdf), T, _ptr(spheres),
+        _lib.check(self._lib.pcdf_ctx_query_cost_backward(self._h, g, _ptr(sdf), T, _ptr(spheres),
                                                           _ptr(tidx), N, float(eps), _ptr(grad_h), _ptr(gc),
                                                           _ptr(gr)), "pcdf_ctx_query_cost_backward")
         return gc, gr
@@ -749,7 +781,7 @@ class Batch:
         _lib.check(self._lib.pcdf_batch_workspace_bytes(h, ctypes.byref(nbytes)), "pcdf_batch_workspace_bytes")
         self.workspace = _workspace(nbytes.value, self.device)
         _lib.check(self._lib.pcdf_batch_upload(h, _ptr(self.workspace), self.workspace.numel(),
-                                               ctypes.c_void_p(_stream(self.device))), "pcdf_batch_upload")
+                                               _stream(self.device)), "pcdf_batch_upload")
 
     @property
     def tiles(self):
@@ -758,12 +790,12 @@ class Batch:
         return (t.row_rows, t.dyn_slices, t.comp_t)
 
     def run(self):
-        _lib.check(self._lib.pcdf_batch_run(self._h, _ptr(self.workspace), ctypes.c_void_p(_stream(self.device))),
+        _lib.check(self._lib.pcdf_batch_run(self._h, _ptr(self.workspace), _stream(self.device)),
                    "pcdf_batch_run")
 
     def error(self) -> int:
         code = ctypes.c_int32(0)
-        _lib.check(self._lib.pcdf_batch_error(self._h, _ptr(self.workspace), ctypes.c_void_p(_stream(self.device)),
+        _lib.check(self._lib.pcdf_batch_error(self._h, _ptr(self.workspace), _stream(self.device),
                                               ctypes.byref(code)), "pcdf_batch_error")
         return code.value
 
@@ -773,7 +805,7 @@ class Batch:
         the next run() then reports PCDF_ETIMEOUT through error()."""
         _lib.check(self._lib.pcdf_batch_block_stage(self._h, int(env), int(stage)), "pcdf_batch_block_stage")
         _lib.check(self._lib.pcdf_batch_upload(self._h, _ptr(self.workspace), self.workspace.numel(),
-                                               ctypes.c_void_p(_stream(self.device))), "pcdf_batch_upload")
+                                               _stream(self.device)), "pcdf_batch_upload")
 
     def close(self):
         if getattr(self, "_h", None):
@@ -811,7 +843,7 @@ def batch_autotune(envs, reps: int = 3, device=None):
     ws = _workspace(nbytes.value, device)
     best = _lib.PcdfBatchTiles()
     ms = ctypes.c_float(0)
-    _lib.check(lib.pcdf_batch_autotune(arr, len(envs), _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(device)),
+    _lib.check(lib.pcdf_batch_autotune(arr, len(envs), _ptr(ws), ws.numel(), _stream(device),
                                        int(reps), ctypes.byref(best), ctypes.byref(ms)), "pcdf_batch_autotune")
     return (best.row_rows, best.dyn_slices, best.comp_t), ms.value
 
@@ -843,7 +875,7 @@ class SurrogateMLP:
         self.reset(seed)
 
     def reset(self, seed: int):
-        _lib.check(self._lib.pcdf_mlp_init(_ptr(self.state), int(seed), ctypes.c_void_p(_stream(self.device))),
+        _lib.check(self._lib.pcdf_mlp_init(_ptr(self.state), int(seed), _stream(self.device)),
                    "pcdf_mlp_init")
         self.step = 0
 
@@ -861,7 +893,7 @@ class SurrogateMLP:
         y = torch.empty(M, dtype=torch.float32, device=self.device)
         ws = self._workspace(M)
         _lib.check(self._lib.pcdf_mlp_forward(_ptr(self.state), _ptr(x), M, _ptr(y), _ptr(ws), ws.numel(),
-                                              ctypes.c_void_p(_stream(self.device))), "pcdf_mlp_forward")
+                                              _stream(self.device)), "pcdf_mlp_forward")
         return y
 
     def infer(self, x: torch.Tensor) -> torch.Tensor:
@@ -871,7 +903,7 @@ class SurrogateMLP:
         M = x.shape[0]
         y = torch.empty(M, dtype=torch.float32, device=self.device)
         _lib.check(self._lib.pcdf_mlp_infer(_ptr(self.state), _ptr(x), M, _ptr(y),
-                                            ctypes.c_void_p(_stream(self.device))), "pcdf_mlp_infer")
+                                            _stream(self.device)), "pcdf_mlp_infer")
         return y
 
     def infer_tc(self, x: torch.Tensor, count: torch.Tensor = None) -> torch.Tensor:
@@ -883,7 +915,7 @@ class SurrogateMLP:
         _need(x, "x", torch.bfloat16)
         M = x.shape[0]
         y = torch.empty(M, dtype=torch.float32, device=self.device)
-        st = ctypes.c_void_p(_stream(self.device))
+        st = _stream(self.device)
         if count is None:
             _lib.check(self._lib.pcdf_mlp_infer_tc(_ptr(self.state), _ptr(x), M, _ptr(y), st), "pcdf_mlp_infer_tc")
         else:
@@ -901,7 +933,7 @@ class SurrogateMLP:
         loss = torch.zeros(1, dtype=torch.float32, device=self.device)
         ws = self._workspace(M)
         _lib.check(self._lib.pcdf_mlp_backward(_ptr(self.state), _ptr(x), _ptr(target), M, _ptr(y), _ptr(loss),
-                                               _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(self.device))),
+                                               _ptr(ws), ws.numel(), _stream(self.device)),
                    "pcdf_mlp_backward")
         return y, loss
 
@@ -927,7 +959,7 @@ class SurrogateMLP:
     def adam(self, lr: float, beta1=0.9, beta2=0.999, eps=1e-8):
         self.step += 1
         _lib.check(self._lib.pcdf_mlp_adam(_ptr(self.state), float(lr), float(beta1), float(beta2), float(eps),
-                                           self.step, ctypes.c_void_p(_stream(self.device))), "pcdf_mlp_adam")
+                                           self.step, _stream(self.device)), "pcdf_mlp_adam")
 
     def train_step(self, x, target, lr):
         _, loss = self.backward(x, target)
@@ -980,9 +1012,9 @@ def surrogate_samples(grid, fields, caps, tf, T, M, seed, near=0.5):
     x = torch.empty((M, MLP_IN_PAD), dtype=torch.bfloat16, device=dev)
     t = torch.empty(M, dtype=torch.float32, device=dev)
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_surrogate_samples(ctypes.byref(g), _ptr(fields), _ptr(caps), _ptr(tf),
+    _lib.check(_lib.load().pcdf_surrogate_samples(g, _ptr(fields), _ptr(caps), _ptr(tf),
                                                   int(fields.shape[0]), int(T), int(M), int(seed), float(near),
-                                                  _ptr(x), _ptr(t), ctypes.c_void_p(_stream(dev))),
+                                                  _ptr(x), _ptr(t), _stream(dev)),
                "pcdf_surrogate_samples")
     return x, t
 
@@ -997,8 +1029,8 @@ def surrogate_features(grid, spheres, tidx, T, caps_dev):
     dev = spheres.device
     x = torch.empty((N * H, MLP_IN_PAD), dtype=torch.bfloat16, device=dev)
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_surrogate_features(ctypes.byref(g), _ptr(spheres), _ptr(tidx), N, int(T), H,
-                                                   _ptr(caps_dev), _ptr(x), ctypes.c_void_p(_stream(dev))),
+    _lib.check(_lib.load().pcdf_surrogate_features(g, _ptr(spheres), _ptr(tidx), N, int(T), H,
+                                                   _ptr(caps_dev), _ptr(x), _stream(dev)),
                "pcdf_surrogate_features")
     return x
 
@@ -1017,13 +1049,13 @@ def surrogate_select(grid, static_sdf, spheres, tidx, T, caps_dev, eps, certifie
     dev = spheres.device
     x = torch.empty((max(N * H, 1), MLP_IN_PAD), dtype=torch.bfloat16, device=dev)
     yi = torch.empty(max(N * H, 1), dtype=torch.int32, device=dev)
-    cnt = torch.zeros(1, dtype=torch.int32, device=dev)
+    cnt = torch.empty(1, dtype=torch.int32, device=dev)  # the call zeroes it
     bounds = torch.empty((max(N, 1), 2), dtype=torch.float32, device=dev)
     g = _cgrid(grid)
-    _lib.check(_lib.load().pcdf_surrogate_select(ctypes.byref(g), _ptr(static_sdf), _ptr(spheres), _ptr(tidx), N,
+    _lib.check(_lib.load().pcdf_surrogate_select(g, _ptr(static_sdf), _ptr(spheres), _ptr(tidx), N,
                                                  int(T), H, _ptr(caps_dev), float(eps), 0 if certified else 1,
                                                  _ptr(x), _ptr(yi), _ptr(cnt), _ptr(bounds),
-                                                 ctypes.c_void_p(_stream(dev))), "pcdf_surrogate_select")
+                                                 _stream(dev)), "pcdf_surrogate_select")
     if not sync:
         return x, yi, cnt, bounds
     return x[: int(cnt.item())], yi, bounds
@@ -1045,21 +1077,22 @@ def surrogate_finish(grid, static_sq, static_sdf, spheres, tidx, T, caps, y, eps
     dev = spheres.device
     h = torch.empty(tidx.shape, dtype=torch.float32, device=dev)
     d = torch.empty(tidx.shape, dtype=torch.float32, device=dev)
-    nfb = torch.zeros(1, dtype=torch.int32, device=dev)
+    # written by the call unless there is no query
+    nfb = (torch.empty if N else torch.zeros)(1, dtype=torch.int32, device=dev)
     n = ctypes.c_size_t(0)
     lib = _lib.load()
     _lib.check(lib.pcdf_surrogate_finish_workspace_bytes(int(T), H, N, ctypes.byref(n)), "surrogate workspace")
     ws = _workspace(n.value, dev)
     g = _cgrid(grid)
     cp = caps.ctypes.data_as(ctypes.c_void_p)
-    tail = (float(eps), float(band), _ptr(h), _ptr(d), _ptr(nfb), _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(dev)))
+    tail = (float(eps), float(band), _ptr(h), _ptr(d), _ptr(nfb), _ptr(ws), ws.numel(), _stream(dev))
     if comp_workspace is None:
-        _lib.check(lib.pcdf_surrogate_finish(ctypes.byref(g), _ptr(static_sq), _ptr(static_sdf), _ptr(spheres),
+        _lib.check(lib.pcdf_surrogate_finish(g, _ptr(static_sq), _ptr(static_sdf), _ptr(spheres),
                                              _ptr(tidx), N, int(T), H, cp, _ptr(y), _ptr(y_index), _ptr(bounds),
                                              *tail), "pcdf_surrogate_finish")
     else:
         _need(comp_workspace, "comp_workspace", torch.uint8)
-        _lib.check(lib.pcdf_surrogate_finish_slab(ctypes.byref(g), _ptr(static_sq), _ptr(static_sdf), _ptr(spheres),
+        _lib.check(lib.pcdf_surrogate_finish_slab(g, _ptr(static_sq), _ptr(static_sdf), _ptr(spheres),
                                                   _ptr(tidx), N, int(T), H, cp, _ptr(comp_workspace),
                                                   comp_workspace.numel(), _ptr(y), _ptr(y_index), _ptr(bounds),
                                                   *tail), "pcdf_surrogate_finish_slab")
@@ -1083,8 +1116,7 @@ def surrogate_step(model, grid, static_sq, static_sdf, spheres, tidx, caps, eps,
     main = torch.cuda.current_stream(dev)
     side = _side_stream(dev)
     side.wait_stream(main)
-    with torch.cuda.stream(side):
-        composite_prepare(grid, caps, comp_workspace)
+    _prepare(grid, caps, comp_workspace, side.cuda_stream)
     comp_workspace.record_stream(side)
     x, yi, cnt, bounds = surrogate_select(grid, static_sdf, spheres, tidx, T, caps_dev, eps, sync=False)
     main.wait_stream(side)

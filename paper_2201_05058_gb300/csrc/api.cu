@@ -243,6 +243,18 @@ int pcdf_query_cost(const pcdf_grid *grid, const float *sdf, int32_t T, const fl
     return e == cudaSuccess ? PCDF_OK : cuda_fail(e, "query");
 }
 
+int pcdf_query_cost_packed(const pcdf_grid *grid, const float *sdf, int32_t T, const float *centres, const float *radii,
+                           const int32_t *tidx, int64_t N, float eps, float *spheres, float *h, void *stream)
+{
+    if (int rc = check_query(grid, sdf, T, spheres, tidx, N))
+        return rc;
+    if (N > 0 && (!centres || !radii || !h))
+        return fail(PCDF_EINVAL, "centres, radii and h must be non-NULL");
+    cudaError_t e = pcdf::launch_query_cost_packed(qgrid(grid), sdf, T, centres, radii, tidx, N, eps, (float4 *)spheres, h,
+                                                   (cudaStream_t)stream);
+    return e == cudaSuccess ? PCDF_OK : cuda_fail(e, "query");
+}
+
 int pcdf_query_cost_backward(const pcdf_grid *grid, const float *sdf, int32_t T, const float *spheres,
                              const int32_t *tidx, int64_t N, float eps, const float *grad_h, float *grad_c,
                              float *grad_r, void *stream)

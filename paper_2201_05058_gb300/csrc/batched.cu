@@ -345,9 +345,14 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
     if (B.smem > 227 * 1024 || B.smem_comp > 227 * 1024)
         return fail(PCDF_EINVAL, "an environment needs %zu bytes of shared memory (limit 227 KB)",
                     std::max(B.smem, B.smem_comp));
-    cudaError_t e = allow_shared(k_batched);
+    cudaFuncAttributes a1, a2;
+    cudaError_t e = cudaFuncGetAttributes(&a1, k_batched);
     if (e == cudaSuccess)
-        e = allow_shared(k_batched_comp);
+        e = cudaFuncGetAttributes(&a2, k_batched_comp);
+    if (e == cudaSuccess)
+        e = allow_shared(k_batched, a1.sharedSizeBytes);
+    if (e == cudaSuccess)
+        e = allow_shared(k_batched_comp, a2.sharedSizeBytes);
     if (e != cudaSuccess)
         return cuda_fail(e, "batched kernel attributes");
     int dev = 0, sms = 0, per_sm = 0, per_sm_comp = 0;

@@ -128,17 +128,15 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
 cudaError_t launch_envelope_i16(const int16_t *in, int32_t *out, int n, int nx, long long ncols,
                                 long long outer_stride, long long stride, cudaStream_t stream);
 
-// Every launch of `kernel` may use all of the SM's shared memory.  The
-// attribute belongs to the kernel, so one value for all calls: a smaller limit
-// set by another thread or plan in between would refuse a launch.
+// Every launch of `kernel` (without static shared memory) may use all of the
+// SM's shared memory.  The attribute belongs to the kernel, so one value for
+// all calls: a smaller limit set by another thread or plan in between would
+// refuse a launch.
+constexpr size_t kMaxShared = 227 * 1024;
 template <class K>
-cudaError_t allow_shared(K kernel)
+cudaError_t allow_shared(K kernel, size_t fixed = 0)
 {
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   227 * 1024 - (int)a.sharedSizeBytes);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxShared - fixed));
 }
 
 // x+y passes of the capsule field over the slab slices zlo .. zlo+S-1 for
@@ -173,6 +171,9 @@ struct QueryGrid {
 cudaError_t launch_query_cost(const QueryGrid &g, const float *sdf, int T, const float4 *spheres,
                               const int32_t *tidx, long long N, float eps, float *h, int32_t *n_oob,
                               cudaStream_t stream);
+cudaError_t launch_query_cost_packed(const QueryGrid &g, const float *sdf, int T, const float *centres,
+                                     const float *radii, const int32_t *tidx, long long N, float eps, float4 *spheres,
+                                     float *h, cudaStream_t stream);
 cudaError_t launch_query_cost_backward(const QueryGrid &g, const float *sdf, int T, const float4 *spheres,
                                        const int32_t *tidx, long long N, float eps, const float *grad_h,
                                        float *grad_c, float *grad_r, cudaStream_t stream);

@@ -7,7 +7,6 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <map>
 #include <vector>
 
 #include "host.h"
@@ -167,21 +166,37 @@ long long slice_key(const CapInfo &c, int k)
     return dz > c.r ? kKeyEmpty : dz;
 }
 
+// The keys of a t's slices lie in one array and are compared through a hash of
+// each, with no allocation per slice: a tree of key vectors here took most of
+// a small call's host time.
 void plan_slab_map(int T, int H, CompositePlan &p)
 {
     p.rep.clear();
     if (p.S <= 0 || p.S > 255 || (long long)T * p.S > kSlabMapMax)
         return;
     p.rep.resize((size_t)T * p.S);
-    std::map<std::vector<long long>, int> first;  // key vector -> first slice of this t holding it
-    std::vector<long long> key(std::max(H, 0));
+    const int n = std::max(H, 0);
+    std::vector<long long> keys((size_t)p.S * n);
+    std::vector<uint64_t> hash(p.S);
+    std::vector<int> firsts;  // the first slice of each kind so far
     for (int t = 0; t < T; ++t) {
-        first.clear();
+        firsts.clear();
         for (int e = 0; e < p.S; ++e) {
-            for (int h = 0; h < H; ++h)
+            long long *key = keys.data() + (size_t)e * n;
+            uint64_t x = 0;
+            for (int h = 0; h < n; ++h) {
                 key[h] = slice_key(p.ci[(size_t)t * H + h], p.zlo + e);
-            const auto it = first.emplace(key, e).first;
-            p.rep[(size_t)t * p.S + e] = (uint8_t)it->second;
+                x = (x ^ (uint64_t)key[h]) * 0x9E3779B97F4A7C15ull;
+                x ^= x >> 29;
+            }
+            hash[e] = x;
+            int rep = e;
+            for (size_t i = firsts.size(); i-- > 0 && rep == e;)  // most slices repeat a recent kind
+                if (hash[firsts[i]] == x && std::equal(key, key + n, keys.data() + (size_t)firsts[i] * n))
+                    rep = firsts[i];
+            if (rep == e)
+                firsts.push_back(e);
+            p.rep[(size_t)t * p.S + e] = (uint8_t)rep;
         }
     }
 }

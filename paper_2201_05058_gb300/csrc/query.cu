@@ -14,14 +14,23 @@ namespace {
 
 __device__ __forceinline__ int time_index(int s, int T) { return min(max(s, 0), T - 1); }
 
+// kPacked: the sphere comes from centres and radii and is written to `spheres`.
+template <bool kPacked>
 __global__ void k_query_cost(const QueryGrid g, const float *__restrict__ sdf, int T,
-                             const float4 *__restrict__ spheres, const int32_t *__restrict__ tidx, long long N,
-                             float eps, float *__restrict__ h, int32_t *__restrict__ n_oob)
+                             const float *__restrict__ centres, const float *__restrict__ radii,
+                             float4 *__restrict__ spheres, const int32_t *__restrict__ tidx, long long N, float eps,
+                             float *__restrict__ h, int32_t *__restrict__ n_oob)
 {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     bool oob = false;
     if (q < N) {
-        const float4 s = __ldg(spheres + q);
+        float4 s;
+        if (kPacked) {
+            s = make_float4(__ldg(centres + 3 * q), __ldg(centres + 3 * q + 1), __ldg(centres + 3 * q + 2), __ldg(radii + q));
+            spheres[q] = s;
+        } else {
+            s = __ldg(spheres + q);
+        }
         const int t = time_index(__ldg(tidx + q), T);
         const long long V = (long long)g.n[0] * g.n[1] * g.n[2];
         const Sample r = trilinear(g, sdf + (PCDF_IN(t, T) ? t : 0) * V, s, false);
@@ -68,7 +77,19 @@ cudaError_t launch_query_cost(const QueryGrid &g, const float *sdf, int T, const
     if (N <= 0)
         return cudaSuccess;
     const long long nblk = (N + 255) / 256;
-    k_query_cost<<<(unsigned)nblk, 256, 0, stream>>>(g, sdf, T, spheres, tidx, N, eps, h, n_oob);
+    k_query_cost<false><<<(unsigned)nblk, 256, 0, stream>>>(g, sdf, T, nullptr, nullptr, const_cast<float4 *>(spheres), tidx,
+                                                            N, eps, h, n_oob);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_query_cost_packed(const QueryGrid &g, const float *sdf, int T, const float *centres,
+                                     const float *radii, const int32_t *tidx, long long N, float eps, float4 *spheres,
+                                     float *h, cudaStream_t stream)
+{
+    if (N <= 0)
+        return cudaSuccess;
+    const long long nblk = (N + 255) / 256;
+    k_query_cost<true><<<(unsigned)nblk, 256, 0, stream>>>(g, sdf, T, centres, radii, spheres, tidx, N, eps, h, nullptr);
     return cudaGetLastError();
 }
 
