@@ -92,8 +92,9 @@ __device__ bool wait_ge(const int *p, int target, int *err)
 __device__ __forceinline__ void run_rows(const BatchEnv &E, int r0, int r1)
 {
     const int lane = threadIdx.x & 31;
-    for (int r = r0 + (threadIdx.x >> 5); r < r1; r += kFirst / 32)
-        full::row_bits_row<0>(E.occ, nullptr, 0, E.nx, E.ny, r, (long long)E.ny * E.nz, E.W, E.bits, E.carry, lane);
+    const int access = full::row_access(E.occ, E.nx), per = full::rows_per_warp(E.W, access);
+    for (int r = r0 + (threadIdx.x >> 5) * per; r < r1; r += kFirst / 32 * per)
+        full::row_bits_rows<0>(E.occ, nullptr, 0, E.nx, E.ny, r, r1, E.ny * E.nz, E.W, E.bits, E.carry, lane, access);
 }
 
 // 3 CTAs of 8 warps per SM: the tile of a 320-voxel axis takes 62 KB

@@ -33,94 +33,6 @@ PCDF_HD bool dominated(int s0, int g0, int s1, int g1, int s2, int g2)
     return (f2 - f1) * (s1 - s0) <= (f1 - f0) * (s2 - s1);
 }
 
-// Forward cursor over an envelope stack in shared memory whose entry q lives
-// at stk[q * stride]; the current and next site are kept in registers.
-// eval(z) requires z to be non-decreasing between calls.
-struct EnvCursor {
-    const uint32_t *stk;
-    int stride, top, q;
-    int s, g, sn, gn;
-    __device__ __forceinline__ EnvCursor(const uint32_t *stk_, int stride_, int top_)
-        : stk(stk_), stride(stride_), top(top_), q(0), s(0), g(0), sn(0), gn(0)
-    {
-        if (top >= 0) {
-            s = site_of(stk[0]);
-            g = gval_of(stk[0]);
-        }
-        if (top >= 1) {
-            sn = site_of(stk[stride]);
-            gn = gval_of(stk[stride]);
-        }
-    }
-    // min over the envelope at z; -1 if the envelope is empty
-    __device__ __forceinline__ int eval(int z)
-    {
-        if (top < 0)
-            return -1;
-        int fc = parab(z, s, g);
-        while (q < top) {
-            const int fn = parab(z, sn, gn);
-            if (fn > fc)
-                break;
-            ++q;
-            s = sn;
-            g = gn;
-            fc = fn;
-            if (q < top) {
-                const uint32_t w = stk[(q + 1) * stride];
-                sn = site_of(w);
-                gn = gval_of(w);
-            }
-        }
-        return fc;
-    }
-    __device__ __forceinline__ bool next_wins(int z) const { return q < top && parab(z, sn, gn) <= parab(z, s, g); }
-    __device__ __forceinline__ void advance()
-    {
-        ++q;
-        s = sn;
-        g = gn;
-        if (q < top) {
-            const uint32_t w = stk[(q + 1) * stride];
-            sn = site_of(w);
-            gn = gval_of(w);
-        }
-    }
-    // out[z * ostride] = eval(z) for z = z0 .. z1 - 1 (the envelope non-empty),
-    // taking the same choices as eval without re-evaluating both parabolas
-    // at every z: with f the current and f' the next parabola, f'(z) - f(z)
-    // falls by 2 (sn - s) per step, so the next site takes over when that
-    // running difference is no longer positive; f itself advances by
-    // 2 (z - s) + 1.
-    __device__ __forceinline__ void fill(int z0, int z1, int32_t *out, long long ostride)
-    {
-        if (z0 >= z1)
-            return;
-        int z = z0;
-        while (next_wins(z))
-            advance();
-        int fc = parab(z, s, g), inc = 2 * (z - s) + 1;
-        int delta = q < top ? parab(z, sn, gn) - fc : INT32_MAX, dd = q < top ? 2 * (sn - s) : 0;
-        int32_t *p = out + (long long)z * ostride;
-        for (; z < z1; ++z) {
-            if (delta <= 0) {
-                advance();
-                while (next_wins(z))
-                    advance();
-                fc = parab(z, s, g);
-                inc = 2 * (z - s) + 1;
-                delta = q < top ? parab(z, sn, gn) - fc : INT32_MAX;
-                dd = q < top ? 2 * (sn - s) : 0;
-            }
-            *p = fc;
-            p += ostride;
-            fc += inc;
-            inc += 2;
-            delta -= dd;
-        }
-    }
-};
-
 // Push site (e, g) onto a stack kept in shared memory (entry q at
 // stk[q * stride]) with the top two entries cached in registers, popping the
 // entries that the new site makes useless.

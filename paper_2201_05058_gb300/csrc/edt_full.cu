@@ -5,7 +5,7 @@
 // translated primitive field).
 //
 // Three launches:
-//   k_row_bits  one warp per row (y, z): the row's occupancy as 32-bit words
+//   k_row_bits  one warp per few rows (y, z): the occupancy as 32-bit words
 //               (bit l of word w: voxel x = 32 w + l) and, per word, the
 //               nearest occupied and free voxel left of it and right of it.
 //   k_edt_xy    one CTA per (slice z, 64 columns): the 1-D distance along x of
@@ -24,18 +24,18 @@
 namespace pcdf {
 namespace {
 
-constexpr int kRowsPerCta = 8;  // k_row_bits: rows (warps) per CTA
+constexpr int kRowWarps = 8;  // k_row_bits: warps per CTA
 constexpr int kThreads = 256;   // k_edt_xy, k_edt_z: 8 warps share the blocks of a tile
 
 template <int kMode>
-__global__ void __launch_bounds__(32 * kRowsPerCta)
+__global__ void __launch_bounds__(32 * kRowWarps)
     k_row_bits(const uint8_t *__restrict__ occ, const __grid_constant__ CapBatch caps, int H, int nx, int ny,
-               long long nrows, int W, uint32_t *__restrict__ bits, uint2 *__restrict__ carry, int vec4)
+               int nrows, int W, uint32_t *__restrict__ bits, uint2 *__restrict__ carry, int access)
 {
-    const long long row = (long long)blockIdx.x * kRowsPerCta + (threadIdx.x >> 5);
+    const int row = ((int)blockIdx.x * kRowWarps + (int)(threadIdx.x >> 5)) * full::rows_per_warp(W, access);
     if (row >= nrows)
         return;  // warp-uniform
-    full::row_bits_row<kMode>(occ, caps.caps, H, nx, ny, row, nrows, W, bits, carry, threadIdx.x & 31, vec4 != 0);
+    full::row_bits_rows<kMode>(occ, caps.caps, H, nx, ny, row, nrows, nrows, W, bits, carry, threadIdx.x & 31, access);
 }
 
 // 46 us for a 256^3 map of 60 boxes (85 us with the stack envelopes it
@@ -83,19 +83,18 @@ cudaError_t launch_full_edt(int mode, const uint8_t *occ, const CapBatch *caps, 
     uint2 *carry = (uint2 *)((char *)ws + co);
     int32_t *mid = (int32_t *)((char *)ws + mo);
     const int W = (nx + 31) / 32;
-    const long long nrows = (long long)ny * nz;
-    const unsigned nb = (unsigned)((nrows + kRowsPerCta - 1) / kRowsPerCta);
-    // occupancy rows of whole 32-bit words: read four bytes per lane
-    const int vec4 = nx % 4 == 0 && ((uintptr_t)occ & 3u) == 0;
+    const int nrows = ny * nz, access = mode == 0 ? full::row_access(occ, nx) : full::kBytes;
+    const int per_cta = kRowWarps * full::rows_per_warp(W, access);
+    const unsigned nb = (unsigned)((nrows + per_cta - 1) / per_cta);
     switch (mode) {
     case 0:
-        k_row_bits<0><<<nb, 32 * kRowsPerCta, 0, st>>>(occ, *caps, H, nx, ny, nrows, W, bits, carry, vec4);
+        k_row_bits<0><<<nb, 32 * kRowWarps, 0, st>>>(occ, *caps, H, nx, ny, nrows, W, bits, carry, access);
         break;
     case 1:
-        k_row_bits<1><<<nb, 32 * kRowsPerCta, 0, st>>>(occ, *caps, H, nx, ny, nrows, W, bits, carry, 0);
+        k_row_bits<1><<<nb, 32 * kRowWarps, 0, st>>>(occ, *caps, H, nx, ny, nrows, W, bits, carry, access);
         break;
     default:
-        k_row_bits<2><<<nb, 32 * kRowsPerCta, 0, st>>>(occ, *caps, H, nx, ny, nrows, W, bits, carry, 0);
+        k_row_bits<2><<<nb, 32 * kRowWarps, 0, st>>>(occ, *caps, H, nx, ny, nrows, W, bits, carry, access);
         break;
     }
     cudaError_t e = cudaGetLastError();

@@ -115,3 +115,12 @@ def test_composite_blocks(nx, ny, nz, T, boxes):
     batch.run()
     assert batch.error() == 0
     assert np.array_equal(batch.comp_sq[0].cpu().numpy(), want)
+
+
+# rows read in 16-byte pieces, several to a warp, the last warp not full
+@pytest.mark.parametrize("shape", [(3, 11, 32), (5, 7, 64), (7, 3, 128), (5, 5, 256), (1, 1, 512), (1, 3, 512), (2, 9, 96), (3, 3, 100)])
+def test_row_words(shape):
+    rng = np.random.default_rng(shape[2])
+    for density in (0.0, 0.02, 0.5, 0.98):
+        occ = (rng.random(shape) < density).astype(np.uint8) * rng.integers(1, 256, shape).astype(np.uint8)
+        check(occ, oracle.edt((occ != 0).astype(np.uint8)))
