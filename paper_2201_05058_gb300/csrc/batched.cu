@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(kFirst, 3)
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_item, s_ok;
     int *head = state, *err = state + 1, *ctr = state + 2;  // ctr[4 * env + stage]
+    blockmin::fill_squares(smem);  // every tile begins with them: once for all items
     for (;;) {
         if (threadIdx.x == 0)
             s_item = atomicAdd(head, 1);
@@ -130,10 +131,10 @@ __global__ void __launch_bounds__(kFirst, 3)
                 run_rows(E, I.a, min(I.a + row_rows, E.ny * E.nz));
                 break;
             case kY:  // slice I.a, columns from 64 I.b
-                full::edt_xy_block<true>(E.bits, E.carry, E.nx, E.ny, E.nz, E.W, I.b, I.a, E.mid, smem);
+                full::edt_xy_block<true, true>(E.bits, E.carry, E.nx, E.ny, E.nz, E.W, I.b, I.a, E.mid, smem);
                 break;
             case kZ:
-                full::edt_z_block<false, true>(E.mid, E.static_sq, nullptr, 0.f, E.nz, (long long)E.nx * E.ny,
+                full::edt_z_block<false, true, true>(E.mid, E.static_sq, nullptr, 0.f, E.nz, (long long)E.nx * E.ny,
                                                (long long)I.a, E.nx * E.ny % 2 == 0, smem);
                 break;
             case kDyn: {  // time I.a, slices from I.b / 16, columns from 64 (I.b % 16)
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(kFirst, 3)
                 for (int s = s0; s < min(s0 + dyn_slices, E.S); ++s) {
                     if (E.rep && E.rep[I.a * E.S + s] != s)
                         continue;  // read from the earlier slice of equal cross-sections
-                    full::capsule_xy_block(E.caps + (long long)I.a * E.H, E.H, E.nx, E.ny, E.zlo + s, I.b & 15,
+                    full::capsule_xy_block<true>(E.caps + (long long)I.a * E.H, E.H, E.nx, E.ny, E.zlo + s, I.b & 15,
                                            E.dyn + ((long long)I.a * E.S + s) * E.nx * E.ny, smem);
                     __syncthreads();
                 }
@@ -310,11 +311,21 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
             rows.push_back({kRow, e, r, 0});
         D.need[kRow] = (nrows + B.tiles.row_rows - 1) / B.tiles.row_rows;
         const int nxb = (g.nx + full::kTileCols - 1) / full::kTileCols;  // column blocks of a slice (<= 8)
+        // slices that repeat an earlier one's cross-sections need no item: most of
+        // an upright human's, and taking an empty item from the queue costs as much
+        // as a small one
+        D.need[kDyn] = 0;
         for (int t = 0; t < U.T; ++t)
-            for (int s = 0; s < p.S; s += B.tiles.dyn_slices)
+            for (int s = 0; s < p.S; s += B.tiles.dyn_slices) {
+                bool any = p.rep.empty();
+                for (int k = s; k < std::min(s + B.tiles.dyn_slices, p.S) && !any; ++k)
+                    any = p.rep[(size_t)t * p.S + k] == k;
+                if (!any)
+                    continue;
                 for (int xb = 0; xb < nxb; ++xb)
                     dyn.push_back({kDyn, e, t, s * 16 + xb});
-        D.need[kDyn] = U.T * ((p.S + B.tiles.dyn_slices - 1) / B.tiles.dyn_slices) * nxb;
+                D.need[kDyn] += nxb;
+            }
         const long long zcols = (long long)g.nx * g.ny;
         for (int z = 0; z < g.nz; ++z)
             for (int x = 0; x < g.nx; x += full::kTileCols)

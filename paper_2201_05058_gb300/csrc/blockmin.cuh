@@ -105,6 +105,16 @@ struct Info {
     __device__ __forceinline__ bool without(bool f) const { return (w.x >> (f ? 26 : 25)) & 1u; }  // no site of O / F
 };
 
+// The squares at the start of a tile (a barrier before they are used).
+__device__ __forceinline__ void fill_squares(uint32_t *sq)
+{
+    for (int i = threadIdx.x; i < kSqWords / 4; i += blockDim.x) {
+        const int d = i / 2 + kSqMin - 4 * (i & 1);
+        reinterpret_cast<uint4 *>(sq)[i] =
+            make_uint4(both(d * d), both((d - 1) * (d - 1)), both((d - 2) * (d - 2)), both((d - 3) * (d - 3)));
+    }
+}
+
 struct Tile {
     uint32_t *sq;      // sq[8 (d - kSqMin) + j] = (d - j)^2 in both halves
     uint2 *info;       // [nb]
@@ -122,15 +132,6 @@ struct Tile {
     __device__ __forceinline__ Tile(uint2 *info_, uint32_t *v_, uint32_t *lo_, int n_, int nb_)
         : sq(nullptr), info(info_), v(v_), lo(lo_), n(n_), nb(nb_)
     {
-    }
-    // before the barrier that ends the stores
-    __device__ __forceinline__ void init() const
-    {
-        for (int i = threadIdx.x; i < kSqWords / 4; i += blockDim.x) {
-            const int d = i / 2 + kSqMin - 4 * (i & 1);
-            reinterpret_cast<uint4 *>(sq)[i] =
-                make_uint4(both(d * d), both((d - 1) * (d - 1)), both((d - 2) * (d - 2)), both((d - 3) * (d - 3)));
-        }
     }
     __device__ __forceinline__ Info about(int b) const { return Info{info[b]}; }
     // One warp records block b, whose values are x.  without(f): the block
