@@ -286,6 +286,13 @@ __device__ __forceinline__ int search16(uint32_t (&best)[kBlk], uint32_t &u, con
 #pragma unroll
     for (int k = 0; k < kBlk; ++k)
         best[k] = part<kF>(src[k * kPitch]);
+    if (kF) {  // next to a free voxel everywhere (single occupied voxels, thin walls): nothing can be nearer
+        const int most = warp_largest(largest(best) & alive);
+        if (most <= 1 && kBlk * (b + 1) <= t.n) {
+            u = 0;
+            return most;
+        }
+    }
     if (!kF && __popc(own) < 5) {
         visit<kF>(best, t.sq, src, 0, own);
     } else {  // most elements count: constant squares

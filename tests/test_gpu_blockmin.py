@@ -124,3 +124,19 @@ def test_row_words(shape):
     for density in (0.0, 0.02, 0.5, 0.98):
         occ = (rng.random(shape) < density).astype(np.uint8) * rng.integers(1, 256, shape).astype(np.uint8)
         check(occ, oracle.edt((occ != 0).astype(np.uint8)))
+
+
+def test_batches_of_different_sizes_side_by_side():
+    """A smaller batch planned later does not lower the shared memory that an
+    earlier, larger one may launch with."""
+    rng = np.random.default_rng(3)
+    made = []
+    for n in (320, 96, 40):
+        grid = scenes.Grid(48, n, 40, 0.05)
+        occ, _ = scenes.boxes_occupancy(grid, 5, rng)
+        caps = scenes.walking_capsules(grid, 1, 2, rng)
+        made.append((pcdf.Batch([(grid, torch.from_numpy(occ).to("cuda"), caps)]), occ, caps))
+    for batch, occ, caps in made:
+        batch.run()
+        assert batch.error() == 0
+        assert np.array_equal(batch.comp_sq[0].cpu().numpy(), oracle.predicted_composite(oracle.edt(occ), caps))
