@@ -1,5 +1,5 @@
-// Lower-envelope pass of the exact EDT along y or z: device code shared by the
-// stand-alone kernel and the batched persistent kernel (sm_103a).
+// Lower-envelope pass of the exact EDT along y or z: device code of the
+// stand-alone kernel (sm_103a).
 //
 // A CTA owns 32 neighbouring columns (consecutive x: every global access of
 // the CTA is one contiguous 128-byte row) and four threads per column, one per
@@ -32,16 +32,6 @@ namespace env {
 constexpr int kCols = 32;   // columns per CTA
 constexpr int kBands = 4;   // threads per column
 
-// Global loads of stage inputs: through the read-only path, or (kCoherent)
-// L2-coherent loads for data written earlier in the same launch.
-template <bool kCoherent, class T>
-__device__ __forceinline__ T load(const T *p)
-{
-    if (kCoherent)
-        return __ldcg(p);
-    return __ldg(p);
-}
-
 __device__ __forceinline__ int32_t widen(int16_t v)
 {
     const int a = v < 0 ? -(int)v : (int)v;
@@ -49,7 +39,6 @@ __device__ __forceinline__ int32_t widen(int16_t v)
         return v < 0 ? -kInf32 : kInf32;
     return v < 0 ? -(a * a) : a * a;
 }
-__device__ __forceinline__ int32_t widen(int32_t v) { return v; }
 
 // The merged envelope of a column: band k contributes the entries in slots
 // [lo_k + st_k, lo_k + st_k + len_k) of the column's tile; global entry q of
@@ -77,22 +66,17 @@ struct Merged {
 static_assert(kBands == 4, "Merged assumes four bands");
 
 // The CTA (kCols * kBands threads) computes columns [col0, col0 + kCols);
-// smem holds kCols * (n + ceil(n / 32)) words.  colmax (non-NULL: every
-// column's largest output value, indexed by column) is written at the end.
-template <typename TIn, bool kSdf, bool kCoherent>
-__device__ __forceinline__ void envelope_tile(const TIn *__restrict__ in, int32_t *__restrict__ out,
-                                              float *__restrict__ sdf, float vox, int n, int nx, long long ncols,
-                                              long long outer_stride, int stride, long long col0, uint32_t *smem,
-                                              int32_t *__restrict__ colmax = nullptr)
+// smem holds kCols * (n + ceil(n / 32)) words.
+__device__ __forceinline__ void envelope_tile(const int16_t *__restrict__ in, int32_t *__restrict__ out, int n, int nx,
+                                              long long ncols, long long outer_stride, int stride, long long col0,
+                                              uint32_t *smem)
 {
     __shared__ int seg[2][kBands][kCols];  // per column and band: first surviving entry, number of entries
-    __shared__ int32_t s_max[kBands][kCols];
-    int32_t mx = INT32_MIN;  // largest value this thread writes
     const int c = threadIdx.x % kCols, band = threadIdx.x / kCols;
     const long long cl = col0 + c;
     const bool live = cl < ncols;
     const long long base = live ? (cl / nx) * outer_stride + (cl % nx) : 0;
-    const TIn *col = in + base;
+    const int16_t *col = in + base;
     uint32_t *tile = smem + c;                                  // element e at tile[e * kCols]
     uint32_t *mk = smem + (size_t)n * kCols + c;                // occupied bits, word w at mk[w * kCols]
     const int nw = (n + 31) >> 5;
@@ -107,7 +91,7 @@ __device__ __forceinline__ void envelope_tile(const TIn *__restrict__ in, int32_
             uint32_t occ = 0;
 #pragma unroll 8
             for (int i = 0; i < cnt; ++i) {
-                const int32_t v = widen(load<kCoherent>(col + (a + i) * stride));
+                const int32_t v = widen(__ldg(col + (a + i) * stride));
                 tile[(a + i) * kCols] = (uint32_t)v;
                 occ |= (uint32_t)(v < 0) << i;
             }
@@ -149,7 +133,7 @@ __device__ __forceinline__ void envelope_tile(const TIn *__restrict__ in, int32_
                     // set O overwrote the slots: restage the values of the targets
                     for (uint32_t m = tgt; m; m &= m - 1) {
                         const int e = (w << 5) + __ffs(m) - 1;
-                        tile[e * kCols] = (uint32_t)widen(load<kCoherent>(col + e * stride));
+                        tile[e * kCols] = (uint32_t)widen(__ldg(col + e * stride));
                     }
                 }
                 for (uint32_t m = tgt | zs; m; m &= m - 1) {
@@ -223,7 +207,6 @@ __device__ __forceinline__ void envelope_tile(const TIn *__restrict__ in, int32_
             Merged M;
             M.init(seg, c, wpb, n);
             int32_t *o = out + base;
-            float *f = kSdf ? sdf + base : nullptr;
             int q = 0, sc = 0, gc = 0, sn = 0, gn = 0;
             if (M.K > 0) {
                 // first entry whose successor is not closer at e0
@@ -274,23 +257,8 @@ __device__ __forceinline__ void envelope_tile(const TIn *__restrict__ in, int32_
                     }
                     r = set == 0 ? r : -r;
                     o[e * stride] = r;
-                    mx = max(mx, r);
-                    if (kSdf)
-                        f[e * stride] = sq_to_sdf_fast(r, vox);
                 }
             }
-        }
-        __syncthreads();
-    }
-    if (colmax) {  // every thread reaches here (no early exits above)
-        s_max[band][c] = mx;
-        __syncthreads();
-        if (band == 0 && live) {
-            int32_t m = s_max[0][c];
-#pragma unroll
-            for (int k = 1; k < kBands; ++k)
-                m = max(m, s_max[k][c]);
-            colmax[cl] = m;
         }
         __syncthreads();
     }
