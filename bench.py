@@ -684,7 +684,7 @@ def run_native(args):
                               out_sq=comp_sq, out_sdf=comp_sdf)
 
     def z_stage(z_events=None):
-        # the composite's z stage alone (k_colmax + k_composite_z, all columns)
+        # the composite's z stage alone (k_composite_z, all columns)
         if z_events:
             z_events[0].record(stream)
         pcdf.composite_finish(static_sq, grid, caps, ws, comp_sq, comp_sdf, static_sdf=static_sdf)
@@ -761,21 +761,20 @@ def run_native(args):
         translated = {"skipped": str(exc)}
 
     # roofline of the dominant stage, timed by the events around
-    # composite_finish (k_colmax, then k_composite_z). Algorithmic bytes of
+    # composite_finish (k_composite_z). Algorithmic bytes of
     # the composite's second stage per the method: the T int32 + T fp32
     # fields out, the dynamic slab intermediate in, the static field (int32)
-    # in once. The implementation also reads static_sq a second time for the
-    # column maxima (writing one int32 per column) and reads static_sdf so as
-    # to copy instead of taking square roots: implementation_bytes.
+    # in once. The implementation also reads static_sdf so as to copy instead
+    # of taking square roots: implementation_bytes.
     _, S = pcdf.composite_slab(grid, caps)
     V2 = grid.nx * grid.ny
     z_bytes = 8 * T * V + 4 * T * S * V2 + 4 * V
-    z_impl_bytes = (4 * V + 4 * V2) + (8 * V + 4 * T * S * V2 + 8 * T * V)
+    z_impl_bytes = 8 * V + 4 * T * S * V2 + 8 * T * V
     z_avg_ms = float(np.mean(z_ms))
     peak, peak_kind = measured_peaks()
     achieved = z_bytes / (z_avg_ms * 1e-3) / 1e9
     traffic = recorded_traffic("z_stage")
-    roofline = {"bound": "hbm", "kernel": "k_colmax + k_composite_z (composite_finish)", "achieved": achieved,
+    roofline = {"bound": "hbm", "kernel": "k_composite_z (composite_finish)", "achieved": achieved,
                 "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_kind, "traffic": traffic,
                 "algorithmic_bytes": z_bytes, "implementation_bytes": z_impl_bytes,
                 "implementation_frac": z_impl_bytes / (z_avg_ms * 1e-3) / 1e9 / peak, "kernel_ms": z_avg_ms,
@@ -866,7 +865,7 @@ def run_native(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         cpu = cpu_baseline(sc)
 
-    launches_per_step = 6  # static: row, y, z; composite: capsule x+y, column maxima, fused z
+    launches_per_step = 5  # static: row words, x+y, z; composite: capsule x+y, fused z
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": "Gvox/s", "n_gpus": world, "steps": args.steps,

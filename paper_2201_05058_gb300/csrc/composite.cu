@@ -9,9 +9,9 @@ namespace {
 
 // Partial fields of the capsules: one CTA per (slab slice, 64 columns, t).
 // 8 warps; like k_edt_xy bound by instruction issue.  3 humans on 256^2, 7
-// distinct slices at each of 20 t: 48 us (111 us with an envelope per column
+// distinct slices at each of 20 t: 40 us (111 us with an envelope per column
 // and thread, whose serial chain left 8 % of the warps active); 4 humans on
-// 161 x 115, T = 9: 23 us (82 us).
+// 161 x 115, T = 9: 17 us (82 us).
 __global__ void __launch_bounds__(256, 4)
     k_dyn_xy(const __grid_constant__ CapBatch caps, const __grid_constant__ SlabMap map, int H, int nx, int ny,
              int zlo, int S, int t0, int32_t *__restrict__ dyn_mid)
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(256, 4)
 
 // CTAs are ordered t-fastest: those of one column block run together and the
 // static block comes from DRAM once.  Three CTAs of 8 warps (80 registers).
-// 256^3, T = 20, 3 humans: 471 us for 2.82 GB of outputs and inputs, 88 % of
+// 256^3, T = 20, 3 humans: 463 us for 2.82 GB of outputs and inputs, 90 % of
 // the measured copy bandwidth (558 us, and 15 us of column maxima, with an
 // envelope per column and thread); 161 x 115 x 83, T = 9: 46 us (88 us).
 template <bool kSq, bool kSdfOut, bool kStaticSdf>

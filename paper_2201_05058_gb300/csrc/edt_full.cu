@@ -38,9 +38,10 @@ __global__ void __launch_bounds__(32 * kRowWarps)
     full::row_bits_rows<kMode>(occ, caps.caps, H, nx, ny, row, nrows, nrows, W, bits, carry, threadIdx.x & 31, access);
 }
 
-// 46 us for a 256^3 map of 60 boxes (85 us with the stack envelopes it
-// replaced), 33 us for 317 x 211 x 97 with speckle: instruction issue (66 %
-// active).  Four CTAs of 64 registers; held to 48 for five it spills (50 us).
+// 43 us for a 256^3 map of 60 boxes (85 us with the stack envelopes it
+// replaced), 32 us for 317 x 211 x 97 with speckle: instruction issue (67 %
+// active).  Four CTAs of 64 registers; held to 48 for five it spills (50 us
+// when four took 46).
 __global__ void __launch_bounds__(kThreads, 4)
     k_edt_xy(const uint32_t *__restrict__ bits, const uint2 *__restrict__ carry, int nx, int ny, int nz, int W,
              int32_t *__restrict__ mid)
@@ -49,8 +50,8 @@ __global__ void __launch_bounds__(kThreads, 4)
     full::edt_xy_block<false>(bits, carry, nx, ny, nz, W, blockIdx.x, blockIdx.y, mid, smem);
 }
 
-// 50 us for the 256^3 map (105 us before): the 12 bytes per voxel alone take
-// 30 us.
+// 42 us for the 256^3 map after k_edt_xy (105 us before): the 12 bytes per
+// voxel alone take 30 us.
 template <bool kSdf>
 __global__ void __launch_bounds__(kThreads, 4)
     k_edt_z(const int32_t *__restrict__ mid, int32_t *__restrict__ sq, float *__restrict__ sdf, float vox, int n,
