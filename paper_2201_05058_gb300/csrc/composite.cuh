@@ -21,11 +21,13 @@
 // loads the static block once and, for each t, starts from the static values
 // and lowers them by the slab elements that can matter: those whose block's
 // least partial plus squared gap lies below the block's largest value.  For
-// most blocks there is none and the static block is stored as it is; no
-// bounds of the static field are needed beforehand.  Where the humans are
-// nearer the float field is the root of the new value, elsewhere the static
-// float field itself.  Voxels inside a human take the distance to the free
-// voxels (set F), from the same tile.  A block left with a value past the
+// most blocks there is none, and no voxel inside a human: the static block is
+// stored as it is; no bounds of the static field are needed beforehand.  Where
+// the humans are nearer the float field is the root of the new value, elsewhere
+// the static float field itself.  Voxels inside a human take the distance to
+// the free voxels (set F), from the same tile, whatever the static map holds
+// there: it is the lower one where a human reaches deeper into a wall or floor
+// than the wall's own depth.  A block left with a value past the
 // 16-bit range is done again in 32 bits from the partials.
 //
 // Bound by the stores: T fields of 8 bytes per voxel.
@@ -413,12 +415,13 @@ struct Composite {
 #pragma unroll 1
             for (int step = 0; step < nt; ++step) {
                 const Tile tl = tile(smem, step, sb);
-                if (reached(tl, sb.first, b, lane, um) || (um >= kFar16 && sb.count)) {
-                    const int c = b - sb.first;
-                    if (c >= 0 && c < sb.count && tl.about(c).occupied())
-                        inside |= 1ull << (i + step);
-                    else
-                        near |= 1ull << (i + step);
+                const int c = b - sb.first;
+                // voxels inside a human come first: the humans' field is
+                // negative there, below any bound and any solid static block
+                if (c >= 0 && c < sb.count && tl.about(c).occupied()) {
+                    inside |= 1ull << (i + step);
+                } else if (reached(tl, sb.first, b, lane, um) || (um >= kFar16 && sb.count)) {
+                    near |= 1ull << (i + step);
                 } else {
                     int32_t *q = B.sq_of(*this, t0 + step);
                     float *g = B.sdf_of(*this, t0 + step);
