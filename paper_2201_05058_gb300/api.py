@@ -34,12 +34,13 @@ class Grid:
 @lru_cache(maxsize=256)
 def _grid_struct(nx, ny, nz, vox, origin) -> _lib.PcdfGrid:
     """The C struct of a grid's values (read only: one for equal grids)."""
-    return _lib.PcdfGrid(int(nx), int(ny), int(nz), float(vox), (ctypes.c_float * 3)(*(float(v) for v in origin)))
+    return _lib.PcdfGrid(nx, ny, nz, vox, (ctypes.c_float * 3)(*origin))
 
 
 def _cgrid(g) -> _lib.PcdfGrid:
+    # plain numbers before the lookup: an array or a tensor is read at each call
     o = getattr(g, "origin", (0.0, 0.0, 0.0))
-    return _grid_struct(g.nx, g.ny, g.nz, g.vox, o if type(o) is tuple else tuple(float(v) for v in o))
+    return _grid_struct(int(g.nx), int(g.ny), int(g.nz), float(g.vox), tuple(map(float, o)))
 
 
 def _shape(g):
