@@ -47,8 +47,10 @@ def _shape(g):
     return (int(g.nz), int(g.ny), int(g.nx))
 
 
-def _stream(dev: torch.device) -> int:
-    return torch.cuda.current_stream(dev).cuda_stream if dev.index is None else _raw_stream(dev.index)
+def _stream(dev) -> int:
+    """Current stream of a device, as the caller names it (torch.device, text or number)."""
+    i = dev.index if type(dev) is torch.device else None
+    return torch.cuda.current_stream(dev).cuda_stream if i is None else _raw_stream(i)
 
 
 # the current stream's handle without a Stream object around it
