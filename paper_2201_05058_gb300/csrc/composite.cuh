@@ -195,7 +195,7 @@ struct Composite {
     {
         uint32_t *w = smem + step * slab_words(zlo, S, nz);
         uint32_t *v = w + (2 * sb.count + 3) / 4 * 4;
-        return Tile(reinterpret_cast<uint2 *>(w), v, v + sb.count * kPitch * kBlk, nz, sb.count);
+        return Tile(reinterpret_cast<uint2 *>(w), nullptr, v, v + sb.count * kPitch * kBlk, nz, sb.count);
     }
 
     // Bound of slab block q for block c (both counted from the tile's first).
@@ -375,7 +375,7 @@ struct Composite {
                     sign |= v[k];
                     dst[k * kPitch] = v[k];
                 }
-                tl.record(Q, lane, v, __any_sync(0xffffffffu, (sign & 0x80008000u) != 0), kFar16, [](bool) { return false; });
+                tl.record(Q, lane, v, __any_sync(0xffffffffu, (sign & 0x80008000u) != 0));
             }
         }
         __syncthreads();
