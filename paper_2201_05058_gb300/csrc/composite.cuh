@@ -27,8 +27,8 @@
 // the static float field itself.  Voxels inside a human take the distance to
 // the free voxels (set F), from the same tile, whatever the static map holds
 // there: it is the lower one where a human reaches deeper into a wall or floor
-// than the wall's own depth.  A block left with a value past the
-// 16-bit range is done again in 32 bits from the partials.
+// than the wall's own depth.  A block left with a value past the 16-bit range
+// is done in 32 bits from the partials: far_block().
 //
 // Bound by the stores: T fields of 8 bytes per voxel.
 #pragma once
@@ -162,6 +162,39 @@ struct Composite {
             for (int k = 0; k < kBlk; ++k)
                 f[k] = make_float2(sq_to_sdf_fast(s[k].x, vox), sq_to_sdf_fast(s[k].y, vox));
         }
+    }
+
+    // A row of the static field at offset i (in0, in1: whether the lane's
+    // columns take part; others: 0), and of its float field.
+    template <bool kVec>
+    __device__ __forceinline__ int2 row_sq(int i, bool in0, bool in1) const
+    {
+        int2 s = make_int2(0, 0);
+        if (kVec) {
+            if (in0 && PCDF_IN(i + 1, V2 * nz))
+                s = __ldcg(reinterpret_cast<const int2 *>(static_sq + i));
+        } else {
+            if (in0 && PCDF_IN(i, V2 * nz))
+                s.x = __ldcg(static_sq + i);
+            if (in1 && PCDF_IN(i + 32, V2 * nz))
+                s.y = __ldcg(static_sq + i + 32);
+        }
+        return s;
+    }
+    template <bool kVec>
+    __device__ __forceinline__ float2 row_sdf(int i, bool in0, bool in1) const
+    {
+        float2 f = make_float2(0.f, 0.f);
+        if (kVec) {
+            if ((in0 || in1) && PCDF_IN(i + 1, V2 * nz))
+                f = __ldcg(reinterpret_cast<const float2 *>(static_sdf + i));
+        } else {
+            if (in0 && PCDF_IN(i, V2 * nz))
+                f.x = __ldcg(static_sdf + i);
+            if (in1 && PCDF_IN(i + 32, V2 * nz))
+                f.y = __ldcg(static_sdf + i + 32);
+        }
+        return f;
     }
 
     // A row of the output at offset i (in0, in1: whether the lane's columns take part).
@@ -401,7 +434,7 @@ struct Composite {
         // blocks with voxels inside a human.  In one loop the compiler's code
         // for the rare paths slowed the others (366 M instead of 214 M
         // instructions at 256^3, T = 20).
-        unsigned long long near = 0, inside = 0, far = 0;  // bit kMaxSteps * block + step
+        unsigned long long near = 0, inside = 0, far = 0, deep = 0;  // bit kMaxSteps * block + step
         for (int b = wid, i = 0; kBlk * b < nz; b += nw, i += kMaxSteps) {
             const Block<kVec> B(*this, b, o, live);
             int2 s[kBlk];
@@ -420,8 +453,10 @@ struct Composite {
                 // negative there, below any bound and any solid static block
                 if (c >= 0 && c < sb.count && tl.about(c).occupied()) {
                     inside |= 1ull << (i + step);
-                } else if (reached(tl, sb.first, b, lane, um) || (um >= kFar16 && sb.count)) {
+                } else if (reached(tl, sb.first, b, lane, um)) {
                     near |= 1ull << (i + step);
+                } else if (um >= kFar16 && sb.count) {
+                    far |= 1ull << (i + step);
                 } else {
                     int32_t *q = B.sq_of(*this, t0 + step);
                     float *g = B.sdf_of(*this, t0 + step);
@@ -489,7 +524,7 @@ struct Composite {
                     fr[k] = kBlk * b + k < nz ? both(kFar16) : 0u;
                 lower<true>(fr, uf, umf, alive, tl, sb.first, b, lane);
                 if (um >= kFar16 || umf >= kFar16) {
-                    far |= 1ull << (i + step);
+                    deep |= 1ull << (i + step);
                     continue;
                 }
                 int32_t *q = B.sq_of(*this, t0 + step);
@@ -506,15 +541,121 @@ struct Composite {
             }
         }
 
-        // rare, and written for few registers: a search with arrays here slowed
-        // the loop above (356 M instead of 254 M instructions at 256^3, T = 20)
+        // voxels inside a human in a block that reaches out of the 16-bit
+        // range: rare, and written for few registers (a search with arrays here
+        // slowed the loops above: 356 M instead of 254 M instructions at 256^3,
+        // T = 20)
+        for (int b = wid; deep; b += nw, deep >>= kMaxSteps)
+#pragma unroll 1
+            for (int step = 0; step < nt; ++step)
+                if ((deep >> step) & 1u)
+#pragma unroll 1
+                    for (int k = 0; k < kBlk && kBlk * b + k < nz; ++k)
+                        whole_column<kVec>(t0 + step, kBlk * b + k, o, live);
+        // blocks 177 voxels or more from the humans and the map: an empty map, or one with few obstacles
         for (int b = wid; far; b += nw, far >>= kMaxSteps)
 #pragma unroll 1
             for (int step = 0; step < nt; ++step)
                 if ((far >> step) & 1u)
+                    far_block<kVec>(t0 + step, b, o, live);
+    }
+
+    // Block b of time t, none of whose voxels is inside a human, in 32 bits and
+    // without the tile: the slab's runs of slices of equal cross-sections (an
+    // upright human between its ends is one) one by one, those that can lower a
+    // column.  An empty map of 256^3, T = 8 and one human (most of the field is
+    // 177 voxels or more from the human): 0.58 ms, where the whole slab for
+    // every voxel took 5.6; on a map of five boxes 0.23 ms.  Issue and latency
+    // of about 1,200 instructions per block and step.
+    template <bool kVec>
+    __device__ __forceinline__ void far_block(int t, int b, int o, const bool (&live)[2]) const
+    {
+        const int lane = threadIdx.x & 31;
+        const Block<kVec> B(*this, b, o, live);
+        int p[kBlk], q[kBlk];  // the least of the static values (negative ones as 0) and the distance to the humans
+#pragma unroll
+        for (int k = 0; k < kBlk; ++k) {
+            const int2 s = row_sq<kVec>(B.at + k * V2, k < B.r0, k < B.r1);
+            p[k] = min(max(s.x, 0), kCap32);
+            q[k] = min(max(s.y, 0), kCap32);
+        }
+        int u0 = largest32(p), u1 = largest32(q);
+        bool lower = false;  // some run lies below in some column
+        const int32_t *src = dyn_mid + ((long long)t * S * V2 + o);
+        // 32 slices at a time, from the middle one's run (the humans' trunks: the least in most columns)
+        const int words = (S + 31) / 32, mid = S / 2, z0 = kBlk * b;
+        for (int n = 0; n < words; ++n) {
+            const int w = mid / 32 + n, e0 = 32 * (w < words ? w : w - words), count = min(S - e0, 32);
+            const int slot = lane < count ? stored(t, e0 + lane) : -1, before = __shfl_up_sync(0xffffffffu, slot, 1);
+            const uint32_t starts = __ballot_sync(0xffffffffu, lane < count && (lane == 0 || slot != before));
+            auto get = [&](int i, int &v0, int &v1) {
+                v0 = v1 = kInf32;
+                const int at = __shfl_sync(0xffffffffu, slot, i);
+                if (!live[0] || !PCDF_IN(at, S) || !PCDF_IN(o, V2))
+                    return;
+                const int32_t *from = src + at * V2;  // a slab holds less than 2^31 values
+                if (kVec) {
+                    const int2 v = __ldcg(reinterpret_cast<const int2 *>(from));
+                    v0 = v.x;
+                    v1 = v.y;
+                } else {
+                    v0 = __ldcg(from);
+                    if (live[1] && PCDF_IN(o + 32, V2))
+                        v1 = __ldcg(from + 32);
+                }
+            };
+            int i = n == 0 ? 31 - __clz(starts & ((2u << (mid & 31)) - 1u)) : 0, a0, a1;
+            uint32_t todo = starts & ~(1u << i);
+            get(i, a0, a1);
 #pragma unroll 1
-                    for (int k = 0; k < kBlk && kBlk * b + k < nz; ++k)
-                        whole_column<kVec>(t0 + step, kBlk * b + k, o, live);
+            for (;;) {  // warp-uniform; the next run's load in flight (two of them cost the batch kernel spills)
+                const int next = __ffs(todo) - 1;
+                int v0 = 0, v1 = 0;
+                if (next >= 0)
+                    get(next, v0, v1);
+                todo &= todo - 1;
+                const uint32_t above = starts & (0xfffffffeu << i);
+                const int za = zlo + e0 + i, zb = zlo + e0 + (above ? __ffs(above) - 2 : count - 1);
+                const int g0 = min(max(a0, 0), kCap32), g1 = min(max(a1, 0), kCap32);
+                const int gap = max(max(za - (z0 + kBlk - 1), z0 - zb), 0);
+                if (__any_sync(0xffffffffu, g0 + gap * gap < u0 || g1 + gap * gap < u1)) {
+                    lower = true;
+#pragma unroll
+                    for (int k = 0; k < kBlk; ++k) {
+                        const int d = max(max(za - (z0 + k), z0 + k - zb), 0);
+                        p[k] = __viaddmin_s32(g0, d * d, p[k]);
+                        q[k] = __viaddmin_s32(g1, d * d, q[k]);
+                    }
+                    u0 = largest32(p);
+                    u1 = largest32(q);
+                }
+                if (next < 0)
+                    break;
+                i = next;
+                a0 = v0;
+                a1 = v1;
+            }
+        }
+        int32_t *g = B.sq_of(*this, t);
+        float *h = B.sdf_of(*this, t);
+#pragma unroll
+        for (int k = 0; k < kBlk; ++k, g += kSq ? V2 : 0, h += kSdfOut ? V2 : 0) {
+            const int i = B.at + k * V2;
+            const bool in0 = k < B.r0, in1 = k < B.r1;
+            int2 s = row_sq<kVec>(i, in0, in1);
+            float2 f = make_float2(0.f, 0.f);
+            if (kStaticSdf)
+                f = row_sdf<kVec>(i, in0, in1);
+            else if (kSdfOut)
+                f = make_float2(sq_to_sdf_fast(s.x, vox), sq_to_sdf_fast(s.y, vox));
+            if (lower) {  // warp-uniform
+                const bool n0 = p[k] < s.x && p[k] < kCap32, n1 = q[k] < s.y && q[k] < kCap32;
+                s = make_int2(n0 ? p[k] : s.x, n1 ? q[k] : s.y);
+                if (kSdfOut)
+                    f = make_float2(n0 ? full::root_near(p[k], vox) : f.x, n1 ? full::root_near(q[k], vox) : f.y);
+            }
+            store<kVec>(g, h, i, in0, in1, s, f);
+        }
     }
 
     // Slice z of time t in 32 bits: both sets over the whole slab.
