@@ -166,9 +166,10 @@ long long slice_key(const CapInfo &c, int k)
     return dz > c.r ? kKeyEmpty : dz;
 }
 
-// The keys of a t's slices lie in one array and are compared through a hash of
-// each, with no allocation per slice: a tree of key vectors here took most of
-// a small call's host time.
+// The keys of a t's slices lie in one array and are found through a table of
+// their hashes, with no allocation per slice: a tree of key vectors here took
+// most of a small call's host time, a scan of the slices so far twice the
+// tree's where 255 slices all differ (3 tilted humans, T = 16: 850 us).
 void plan_slab_map(int T, int H, CompositePlan &p)
 {
     p.rep.clear();
@@ -178,9 +179,10 @@ void plan_slab_map(int T, int H, CompositePlan &p)
     const int n = std::max(H, 0);
     std::vector<long long> keys((size_t)p.S * n);
     std::vector<uint64_t> hash(p.S);
-    std::vector<int> firsts;  // the first slice of each kind so far
+    constexpr uint32_t kSlots = 512;  // twice the slices at most: a probe ends soon
+    int16_t first[kSlots];            // the first slice of each kind so far (-1: none), by its hash
     for (int t = 0; t < T; ++t) {
-        firsts.clear();
+        std::fill(first, first + kSlots, (int16_t)-1);
         for (int e = 0; e < p.S; ++e) {
             long long *key = keys.data() + (size_t)e * n;
             uint64_t x = 0;
@@ -190,12 +192,12 @@ void plan_slab_map(int T, int H, CompositePlan &p)
                 x ^= x >> 29;
             }
             hash[e] = x;
-            int rep = e;
-            for (size_t i = firsts.size(); i-- > 0 && rep == e;)  // most slices repeat a recent kind
-                if (hash[firsts[i]] == x && std::equal(key, key + n, keys.data() + (size_t)firsts[i] * n))
-                    rep = firsts[i];
-            if (rep == e)
-                firsts.push_back(e);
+            uint32_t at = (uint32_t)(x >> 32) % kSlots;
+            while (first[at] >= 0 && !(hash[first[at]] == x && std::equal(key, key + n, keys.data() + (size_t)first[at] * n)))
+                at = (at + 1) % kSlots;
+            if (first[at] < 0)
+                first[at] = (int16_t)e;
+            const int rep = first[at];
             p.rep[(size_t)t * p.S + e] = (uint8_t)rep;
         }
     }
