@@ -386,7 +386,8 @@ typedef struct pcdf_env {
 typedef struct pcdf_batch_tiles {
     int32_t row_rows;   /* rows per row-pass item (<= 0: 32) */
     int32_t dyn_slices; /* slab slices per capsule-field item (<= 0: 1) */
-    int32_t comp_t;     /* time steps per composite item (<= 0: 1) */
+    int32_t comp_t;     /* time steps per composite item (<= 0: 1; rounded up
+                           to whole runs of those that share their reads) */
 } pcdf_batch_tiles;
 
 typedef struct pcdf_batch pcdf_batch;

@@ -47,9 +47,10 @@ struct BatchItem {
 struct BatchEnv {
     int nx, ny, nz, T, H, zlo, S, W;
     float vox;
-    int need[4];  // items of the row, y, z and capsule stages
+    int need[3];  // items of the row, y and z stages
     int vec;      // two columns in 8 bytes (composite items)
     int steps;    // time steps that a composite CTA takes together
+    int group;    // and those of a composite item: a multiple
     const uint8_t *occ;
     int32_t *comp_sq;
     uint32_t *bits;   // row words, [nz][ny][W]
@@ -97,11 +98,11 @@ __device__ __forceinline__ void run_rows(const BatchEnv &E, int r0, int r1)
         full::row_bits_rows<0>(E.occ, nullptr, 0, E.nx, E.ny, r, r1, E.ny * E.nz, E.W, E.bits, E.carry, lane, access);
 }
 
-// 3 CTAs of 8 warps per SM: the tile of a 320-voxel axis takes 62 KB.  0.78 ms
+// 3 CTAs of 8 warps per SM: the tile of a 320-voxel axis takes 63 KB.  0.71 ms
 // for 16 environments (60 M static voxels, 72 M of distinct capsule slices).
 __global__ void __launch_bounds__(kFirst, 3)
     k_batched(const BatchEnv *__restrict__ envs, const BatchItem *__restrict__ items, int n_items, int *state,
-              int row_rows, int dyn_slices, int comp_t)
+              int row_rows, int dyn_slices)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_item, s_ok;
@@ -163,16 +164,14 @@ __global__ void __launch_bounds__(kFirst, 3)
 
 // The composite items, after every static and capsule item has finished (the
 // previous launch on the stream): item (env, t, column block) computes time
-// steps t .. t + comp_t - 1 of 64 consecutive columns.  The items of a column
-// block follow one another, so a CTA takes `take` items at once and computes
-// those of one column block together, E.steps time steps at a time, reading
-// the static block once for them.  Nothing to wait for; if a dependency wait
-// of the first launch expired, the items are skipped.  1.33 ms for the
-// 16 environments (888 M voxel fields) whose stores alone take 0.52 ms; the
-// envelope per column it replaced took 1.75 ms, 8 warps per CTA take 1.52.
+// steps t .. t + E.group - 1 of 64 consecutive columns, E.steps at a time,
+// reading the static block once for them.  Nothing to wait for; if a
+// dependency wait of the first launch expired, the items are skipped.  1.30 ms
+// for the 16 environments (888 M voxel fields) whose stores alone take 0.52 ms;
+// the envelope per column it replaced took 1.75 ms, 8 warps per CTA take 1.52.
 __global__ void __launch_bounds__(kSecond, 6)
     k_batched_comp(const BatchEnv *__restrict__ envs, const BatchItem *__restrict__ items, int n_items,
-                   const int *__restrict__ err, int *head, int comp_t, int take)
+                   const int *__restrict__ err, int *head)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_item;
@@ -180,27 +179,20 @@ __global__ void __launch_bounds__(kSecond, 6)
         return;  // uniform: every thread reads the same word
     for (;;) {
         if (threadIdx.x == 0)
-            s_item = atomicAdd(head, take);
+            s_item = atomicAdd(head, 1);
         __syncthreads();
-        const int it = s_item, end = min(it + take, n_items);
+        const int it = s_item;
         if (it >= n_items)
             break;
-        for (int i = it; i < end;) {
-            const BatchItem I = items[i];
-            const BatchEnv &E = envs[I.env];
-            int j = i + 1;  // the items of this column block among those taken
-            while (j < end && items[j].env == I.env && items[j].b == I.b)
-                ++j;
-            const int t1 = min(I.a + (j - i) * comp_t, E.T);
-            const comp::Composite<true, false, false> c = {E.static_sq, nullptr, E.dyn, E.rep, E.comp_sq, nullptr,
-                                                           E.nx * E.ny, E.nz, E.zlo, E.S, E.vox, E.vec != 0};
-            for (int t = I.a; t < t1; t += E.steps) {
-                c.run(t, min(E.steps, t1 - t), (long long)I.b, smem);
-                __syncthreads();
-            }
-            i = j;
+        const BatchItem I = items[it];
+        const BatchEnv &E = envs[I.env];
+        const int t1 = min(I.a + E.group, E.T);
+        const comp::Composite<true, false, false> c = {E.static_sq, nullptr, E.dyn, E.rep, E.comp_sq, nullptr,
+                                                       E.nx * E.ny, E.nz, E.zlo, E.S, E.vox, E.vec != 0};
+        for (int t = I.a; t < t1; t += E.steps) {
+            c.run(t, min(E.steps, t1 - t), (long long)I.b, smem);
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
@@ -311,6 +303,9 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         D.W = (g.nx + 31) / 32;
         D.vox = g.vox;
         D.steps = comp::steps_per_cta(p.zlo, p.S, g.nz, U.T, kCompShared);
+        // whole runs of the steps that a CTA takes together (items of comp_t = 1,
+        // taken four at a time, split them: 9 steps as 3 + 1 + 3 + 1 + 1)
+        D.group = (std::max(B.tiles.comp_t, 1) + D.steps - 1) / D.steps * D.steps;
         words_comp = std::max(words_comp, D.steps * comp::slab_words(p.zlo, p.S, g.nz));
         const int nrows = g.ny * g.nz;
         for (int r = 0; r < nrows; r += B.tiles.row_rows)
@@ -320,7 +315,6 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         // slices that repeat an earlier one's cross-sections need no item: most of
         // an upright human's, and taking an empty item from the queue costs as much
         // as a small one
-        D.need[kDyn] = 0;
         for (int t = 0; t < U.T; ++t)
             for (int s = 0; s < p.S; s += B.tiles.dyn_slices) {
                 bool any = p.rep.empty();
@@ -330,7 +324,6 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
                     continue;
                 for (int xb = 0; xb < nxb; ++xb)
                     dyn.push_back({kDyn, e, t, s * 16 + xb});
-                D.need[kDyn] += nxb;
             }
         const long long zcols = (long long)g.nx * g.ny;
         for (int z = 0; z < g.nz; ++z)
@@ -343,7 +336,7 @@ int build_plan(const pcdf_env *envs, int n_env, const pcdf_batch_tiles *tiles, p
         // composite items t-fastest within a column block: the blocks of one
         // column range run together and share the static column in L2
         for (long long c = 0; c < zcols; c += full::kTileCols)
-            for (int t = 0; t < U.T; t += B.tiles.comp_t)
+            for (int t = 0; t < U.T; t += D.group)
                 comps.push_back({kComp, e, t, (int)c});
     }
     B.items.clear();
@@ -492,14 +485,13 @@ int pcdf_batch_run(const pcdf_batch *b, void *workspace, void *stream)
     const BatchEnv *desc = (const BatchEnv *)(ws + b->off_desc);
     const BatchItem *items = (const BatchItem *)(ws + b->off_items);
     k_batched<<<b->blocks, kFirst, b->smem, st>>>(desc, items, b->n_first, state, b->tiles.row_rows,
-                                                   b->tiles.dyn_slices, b->tiles.comp_t);
+                                                  b->tiles.dyn_slices);
     err = cudaGetLastError();
     if (err != cudaSuccess)
         return cuda_fail(err, "batched launch");
     const int n_comp = (int)b->items.size() - b->n_first;
-    const int take = std::max(1, comp::kMaxSteps / b->tiles.comp_t);
-    k_batched_comp<<<b->blocks_comp, kSecond, b->smem_comp, st>>>(
-        desc, items + b->n_first, n_comp, state + 1, state + 2 + 4 * b->n_env, b->tiles.comp_t, take);
+    k_batched_comp<<<b->blocks_comp, kSecond, b->smem_comp, st>>>(desc, items + b->n_first, n_comp, state + 1,
+                                                                  state + 2 + 4 * b->n_env);
     err = cudaGetLastError();
     return err == cudaSuccess ? PCDF_OK : cuda_fail(err, "batched composite launch");
 }
