@@ -121,6 +121,24 @@ def sources_sha(names):
     return h.hexdigest()[:16]
 
 
+def distinct_slices(caps, zlo: int, S: int) -> int:
+    """Slab slices, over all time steps, that the capsule pass computes: one of
+    those of a time step where every upright capsule has the same cross-section
+    (the distance to the nearer cap centre, 0 between the two); a slanted
+    capsule has one of its own in every slice."""
+    n = 0
+    for step in caps:
+        kinds = set()
+        for z in range(zlo, zlo + S):
+            p, key = 16 * z + 8, []
+            for ax, ay, az, bx, by, bz, r in step.tolist():
+                d = max(min(az, bz) - p, p - max(az, bz), 0)
+                key.append(z if (ax, ay) != (bx, by) else -1 if d > r else d)
+            kinds.add(tuple(key))
+        n += len(kinds)
+    return n
+
+
 def recorded_traffic(kernel: str):
     """DRAM bytes per launch of `kernel` from the committed ncu summary
     (profiles/traffic.txt: one line per kernel or stage, `name sources=a,b
@@ -765,11 +783,12 @@ def run_native(args):
     # the composite's second stage per the method: the T int32 + T fp32
     # fields out, the dynamic slab intermediate in, the static field (int32)
     # in once. The implementation also reads static_sdf so as to copy instead
-    # of taking square roots: implementation_bytes.
-    _, S = pcdf.composite_slab(grid, caps)
+    # of taking square roots, and of the slab only the slices whose
+    # cross-sections differ: implementation_bytes.
+    zlo, S = pcdf.composite_slab(grid, caps)
     V2 = grid.nx * grid.ny
     z_bytes = 8 * T * V + 4 * T * S * V2 + 4 * V
-    z_impl_bytes = 8 * V + 4 * T * S * V2 + 8 * T * V
+    z_impl_bytes = 8 * V + 4 * distinct_slices(caps, zlo, S) * V2 + 8 * T * V
     z_avg_ms = float(np.mean(z_ms))
     peak, peak_kind = measured_peaks()
     achieved = z_bytes / (z_avg_ms * 1e-3) / 1e9

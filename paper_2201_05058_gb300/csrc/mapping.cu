@@ -180,7 +180,7 @@ constexpr int kBZ = 8, kBHZ = kBZ + 2, kBThreads = 256;
 
 // nx a multiple of 16, both maps aligned to 16 bytes.
 // thresh: least count, the voxel itself among it, that keeps an occupied voxel.
-// Bound by the loads of its tiles (1.6 times the map, the halo from L2): 13.4 us
+// Bound by the loads of its tiles (1.6 times the map, the halo from L2): 12 us
 // at 256^3 (31.5 us with byte-wise counts in shared memory; 2 bytes per voxel
 // take 5).
 template <int kBW>

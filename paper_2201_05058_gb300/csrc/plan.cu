@@ -235,7 +235,10 @@ int plan_composite(const pcdf_grid *grid, int T, int H, const int32_t *caps, Com
         p.run_rows = std::max(p.run_rows, ext);
     }
     // beyond this bound on the capsules' rows the generic row and y passes
-    // run instead, and batches refuse the environment
+    // run instead, and batches refuse the environment.  It is older than the
+    // present capsule pass, which would fit (at most 225 KB of shared memory):
+    // kept so that the same requests take the same route and the same
+    // environments are refused
     const size_t cap = (size_t)std::min(p.run_rows + 2 * H + 2, grid->ny + 2);
     p.fused = ((size_t)grid->ny * (H + 1) + cap * 128) * 4 <= 200 * 1024 &&
               pcdf::dyn_xy_words(grid->ny, p.run_rows) * 4 <= 227 * 1024;
